@@ -197,6 +197,8 @@ def pass_bytes(kind, info, R, ncomp_tables=1):
         return R * (vec + u2) + 4 * M
     if kind.startswith("yx_inv"):             # fused y+x slice pass: U2 and X in, Y out
         return R * (u2 + 2 * vec) + 4 * M + N
+    if kind.startswith("slab"):               # y and z transforms over kx slabs: the x-transformed rows, both ways
+        return R * 2 * u1 + oct_
     if kind.startswith("x_fwd"):
         return R * (vec + u1) + 4 * M
     if kind.startswith("y_fwd") or kind.startswith("y_inv"):
@@ -613,6 +615,11 @@ def read_profile(dda, ctx):
     for i in range(n.value):
         out[arr[i].name.decode()] = {"launches": arr[i].launches, "ms": arr[i].total_ms, "units": arr[i].units,
                                      "share": arr[i].total_ms / total if total else 0.0}
+    # the slab pass (y and z transforms in one kernel) is traced as a z pass
+    # with empty y passes, and counted once more under its own name
+    if "slab_c64" in out and out["slab_c64"]["launches"] == out["z_conv_c64"]["launches"]:
+        out["slab_c64"] = out.pop("z_conv_c64")
+        del out["y_fwd_c64"], out["y_inv_c64"]
     return out
 
 
@@ -651,7 +658,7 @@ FUSED_VECTORS_PER_MATVEC = {"bicgstab": 5.5}
 
 
 def matvec_roofline(kstats, info, suffix="c64", rhs_matvecs=None, fused_vectors=0.0):
-    """The whole FFT-convolution matvec (its five passes together) against
+    """The whole FFT-convolution matvec (all its passes together) against
     HBM: algorithmic bytes of all launches of the passes / their total time.
 
     Bytes per launch are pass_bytes (compact vectors of N sites, padded
@@ -665,7 +672,7 @@ def matvec_roofline(kstats, info, suffix="c64", rhs_matvecs=None, fused_vectors=
     sites, P read and written on the whole lattice)."""
     hbm, src = load_peaks()
     kinds = [k for k in kstats if k.endswith(suffix) and pass_bytes(k, info, 1) is not None]
-    if len(kinds) not in (3, 5):   # fused slice passes + z, or the five separate passes
+    if len(kinds) not in (3, 5):   # slab or slice passes, or the five separate passes
         return None
     ms = sum(kstats[k]["ms"] for k in kinds)
     b = 0.0
@@ -679,7 +686,7 @@ def matvec_roofline(kstats, info, suffix="c64", rhs_matvecs=None, fused_vectors=
     b += fused_bytes
     ach = b / (ms / 1e3) / 1e9
     M = (info["Lx"] // 2) * (info["Ly"] // 2) * (info["Lz"] // 2)
-    zk = [k for k in kinds if k.startswith("z_conv")][0]
+    zk = [k for k in kinds if k.startswith(("z_conv", "slab"))][0]
     units = kstats[zk]["units"] if rhs_matvecs is None else rhs_matvecs
     sb = (81 * units + 6 * kstats[zk]["launches"]) * M * s
     sach = sb / (ms / 1e3) / 1e9

@@ -335,6 +335,13 @@ dda_status dda_grad_qabs(dda_ctx* ctx, dda_precision precision, const double* kh
  *  - the y passes (complex64 only, Ly = 128, 192, 256): 0 the plan of the
  *    staged passes, 1 a radix plan with one exchange fewer (8 x 16,
  *    8 x 8 x 3, 16 x 16).
+ * Where no setter below asks for anything, complex64 matvecs whose Ly and Lz
+ * are at most 128 run the slab pass instead: the y and z transforms and the
+ * product in one kernel over the kx planes, between x passes of its own, for
+ * every RHS count and without timing anything (anisotropic materials keep the
+ * passes above).  The queries below still report, and make, the choices the
+ * separate passes would run with; launch tracing counts a slab pass as a z
+ * pass with empty y passes, and once more as "slab_c64".
  * All choices compute the same product; results agree to rounding.  In
  * automatic mode the context times the available choices inside whole
  * matvecs on its own workspace the first time a matvec of a given type and

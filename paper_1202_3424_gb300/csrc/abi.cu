@@ -87,6 +87,7 @@ struct dda_ctx {
     bool prepared = false, has32 = false;
     double kd = 0.0, aeff_lat = 0.0;
     DevMem m_gh64, m_gh32, m_tw64[3], m_tw32[3];
+    DevMem m_ghslab;           // the slab pass's copy (slab.cuh), where that pass is built
     DevMem m_ghdf, m_twdf[3];  // double-float copies for the refinement residual
 
     // workspace
@@ -576,6 +577,27 @@ dda_status pick_schedule(dda_ctx* ctx, int R, bool may_time, PadWork<T>* out, bo
     return DDA_OK;
 }
 
+// The passes of a matvec of R right-hand sides: the slab pass (slab.cuh) where
+// it is built and no setter asks for a schedule of the separate passes (which
+// it replaces), else pick_schedule's choice.  Whole matvecs, separate passes ->
+// slab (sum of the kernels): 96x64x32 ellipsoid, 32 RHS 931 -> 763 us; 64^3
+// sphere, 2 RHS 109 -> 90 us; 48^3, 4 RHS 134 -> 108 us; 32^3, 8 RHS 66 -> 53 us.
+// Anisotropic materials keep the separate passes: solves of strongly absorbing
+// crystals amplify a change of rounding until single elements of P differ by
+// 1e-3 at tolerance 1e-5 (BiCGstab(2), 65 cycles), and their users compare runs.
+template <typename T>
+dda_status choose_passes(dda_ctx* ctx, int R, bool may_time, PadWork<T>* out, bool fused = false) {
+    out->slab = nullptr;
+    if constexpr (std::is_same<T, float>::value) {
+        if (slab_built(ctx->g) && !ctx->aniso && ctx->force_z < 0 && ctx->force_xf < 0 && ctx->force_xi < 0 && ctx->force_y < 0 &&
+            ctx->force_slices == 0) {
+            out->slab = static_cast<const float4*>(ctx->m_ghslab.p);
+            return DDA_OK;
+        }
+    }
+    return pick_schedule<T>(ctx, R, may_time, out, fused);
+}
+
 // y = A x over R RHS in chunks (workspace from ensure_pad<T>).
 template <typename T>
 dda_status run_matvec(dda_ctx* ctx, int R, const cx<T>* x, cx<T>* y, const int* active) {
@@ -587,7 +609,7 @@ dda_status run_matvec(dda_ctx* ctx, int R, const cx<T>* x, cx<T>* y, const int* 
     dda_status zs;
     for (int r0 = 0; r0 < R; r0 += rc) {
         const int rn = std::min(rc, R - r0);
-        if ((zs = pick_schedule<T>(ctx, rn, true, &w)) != DDA_OK) return zs;
+        if ((zs = choose_passes<T>(ctx, rn, true, &w)) != DDA_OK) return zs;
         CU(launch_matvec<T>(ctx->g, rn, x + (int64_t)r0 * n, y + (int64_t)r0 * n, w, ctx->tg,
                             beta_of<T>(ctx) + (int64_t)r0 * BS, BS, ghat_of<T>(ctx), tw_of<T>(ctx),
                             active ? active + r0 : nullptr, ctx->stream));
@@ -651,7 +673,7 @@ dda_status run_matvec_fused(dda_ctx* ctx, int R, int mode, cx<T>* x, cx<T>* y, c
     for (int r0 = 0; r0 < R; r0 += rc) {
         const int rn = std::min(rc, R - r0);
         const int64_t o = (int64_t)r0 * n;
-        if ((zs = pick_schedule<T>(ctx, rn, true, &w, true)) != DDA_OK) return zs;
+        if ((zs = choose_passes<T>(ctx, rn, true, &w, true)) != DDA_OK) return zs;
         FusedKrylov<T> fk;
         fk.mode = mode;
         fk.r = r + o;
@@ -1192,7 +1214,7 @@ dda_status matvec_noalloc(dda_ctx* ctx, int R, const std::vector<double>& k, con
     w.beta_tensor = ctx->aniso;
     CU(cudaMemcpyAsync(d_beta, beta.data(), beta.size() * sizeof(C), cudaMemcpyHostToDevice, ctx->stream));
     dda_status zs;
-    if ((zs = pick_schedule<T>(ctx, R, false, &w)) != DDA_OK) return zs;  // no timing here
+    if ((zs = choose_passes<T>(ctx, R, false, &w)) != DDA_OK) return zs;  // no timing here
     CU(launch_matvec<T>(ctx->g, R, static_cast<const C*>(x_dev), static_cast<C*>(y_dev), w, ctx->tg, d_beta, BS,
                         ghat_of<T>(ctx), tw_of<T>(ctx), nullptr, ctx->stream));
     CU(cudaStreamSynchronize(ctx->stream));
@@ -1269,6 +1291,7 @@ dda_status dda_destroy(dda_ctx* ctx) {
     free_mem(ctx->m_gh64);
     free_mem(ctx->m_gh32);
     free_mem(ctx->m_ghdf);
+    free_mem(ctx->m_ghslab);
     for (int a = 0; a < 3; ++a) {
         free_mem(ctx->m_tw64[a]);
         free_mem(ctx->m_tw32[a]);
@@ -1502,6 +1525,10 @@ dda_status dda_prepare(dda_ctx* ctx, double lambda_vac, double aeff, dda_precisi
         CU(launch_convert_c128_to_c64((const double2*)ctx->m_gh64.p, (float2*)ctx->m_gh32.p, oct, ctx->stream));
         if ((s = ensure(ctx, ctx->m_ghdf, oct * sizeof(cdfl))) != DDA_OK) return s;
         CU(launch_convert_c128_to_df((const double2*)ctx->m_gh64.p, (cdfl*)ctx->m_ghdf.p, oct, ctx->stream));
+        if (slab_built(g)) {
+            if ((s = ensure(ctx, ctx->m_ghslab, slab_green_size(g) * sizeof(float4))) != DDA_OK) return s;
+            CU(launch_slab_green(g, (const double2*)ctx->m_gh64.p, (float4*)ctx->m_ghslab.p, ctx->stream));
+        }
         CU(sync_collect(ctx));
         ctx->has32 = true;
     }

@@ -74,6 +74,9 @@ template <typename T> struct PadWork {
     int xfwd = 0;         // x-forward schedule, see xpass_schedules
     int xinv = 0;         // x-inverse schedule, likewise
     int yvar = 0;         // y-pass radix plan variant, see ypass_schedules
+    // the y and z transforms in one pass over kx slabs (slab.cuh, complex64):
+    // the Green tensor in that pass's layout, or null for the separate passes
+    const float4* slab = nullptr;
     int slices = 1;       // fused x+y slice passes where built (see slice_passes)
     // The 1/alpha table holds 3x3 tensors (anisotropic materials): per RHS
     // [3 rows c][comp][3 columns], so row c of composition comp's tensor is at
@@ -144,6 +147,16 @@ template <typename T>
 cudaError_t launch_slice_inv(const Geom& g, int R, const cx<T>* u2, cx<T>* y, const cx<T>* x, const DevTarget& tg,
                              const cx<T>* beta, int beta_stride, const Twiddles<T>& tw, int* active,
                              const FusedKrylov<T>& fk, cudaStream_t st);
+
+// The slab pass (slab.cuh): built for this grid?  Entries (float4) of its copy
+// of the Green tensor, and the kernel that fills it from the FP64 octant.
+bool slab_built(const Geom& g);
+int64_t slab_green_size(const Geom& g);
+cudaError_t launch_slab_green(const Geom& g, const double2* gh64, float4* out, cudaStream_t st);
+// y = A x through the slab pass (w.slab, w.u2), as launch_matvec_fused.
+cudaError_t launch_slab_matvec(const Geom& g, int R, float2* x, float2* y, const PadWork<float>& w, const DevTarget& tg,
+                               const float2* beta, int beta_stride, const Twiddles<float>& tw, int* active,
+                               const FusedKrylov<float>& fk, cudaStream_t st);
 
 // The z pass alone, in place on u2 (used to time the schedules).
 template <typename T>

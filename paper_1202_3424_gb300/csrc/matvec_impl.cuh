@@ -1173,6 +1173,10 @@ cudaError_t launch_matvec_fused(const Geom& g, int R, cx<T>* x, cx<T>* y, const 
         DDA_DISPATCH_L(g.Lx, LX::template inv, g, R, w.u2, y, x, tg, beta, beta_stride, w.beta_tensor, tw.x, active,
                        fk, w.xinv, st);
     };
+    if constexpr (std::is_same<T, float>::value) {
+        if (w.slab != nullptr)
+            return launch_slab_matvec(g, R, x, y, w, tg, beta, beta_stride, tw, active, fk, st);
+    }
     if (w.slices && !w.beta_tensor && slice_passes<T>(g)) {
         if ((e = launch_slice_fwd<T>(g, R, x, w.u2, tg.site_of, tw, active, fk, st)) != cudaSuccess) return e;
         if ((e = zc()) != cudaSuccess) return e;

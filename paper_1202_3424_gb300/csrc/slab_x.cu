@@ -1,0 +1,129 @@
+// The slab matvec (slab.cuh): its x passes, its copy of the Green tensor, and
+// the launcher.
+#include "slab.h"
+
+#include "slab.cuh"
+
+namespace dda {
+
+namespace {
+
+// Radix plan variant of the warp-local rows (XwPlan): forward, the one with the
+// fewest exchanges through shared memory; inverse, the one with the fewest
+// registers, but for 192 points, where the plan with three exchanges holds the
+// pass at its shared-memory rate (96x64x32 ellipsoid, 32 RHS: 190 us, against
+// 168 us with two).
+template <int LX> constexpr int kPlanFwd = (LX == 128 || LX == 192 || LX == 256) ? 1 : 0;
+template <int LX> constexpr int kPlanInv = LX == 192 ? 1 : 0;
+
+template <int LX>
+cudaError_t xfwd(const Geom& g, int R, float2* x, float2* u, const DevTarget& tg, const float2* tw, const int* active,
+                 const FusedKrylov<float>& fk, cudaStream_t st) {
+    constexpr int V = kPlanFwd<LX>;
+    using PL = XwPlan<LX, V>;
+    const size_t sm = xw_tile_bytes<PL>(xw_rows<PL>()) + (xw_shared_twiddles<LX>() ? LX * sizeof(float2) : 0);
+    const int nrows = g.ny * g.nz;
+    dim3 grid((nrows + xw_rows<PL>() - 1) / xw_rows<PL>(), 3, R);
+    RowMap rm = row_map(g);
+    rm.pitch = nrows;
+    auto go = [&](auto kern) -> cudaError_t {
+        cudaError_t e = allow_smem(kern, sm);
+        if (e != cudaSuccess) return e;
+        PROF_BEGIN(st);
+        kern<<<grid, kXwThreads, sm, st>>>(x, u, rm, tg.site_of, nrows, g.N, tw, active, fwd_vecs(fk));
+        PROF_END(KK_XFWD_C64, R, st);
+        return cudaGetLastError();
+    };
+    if (fk.mode == 0) return go(k_xfwd_w<LX, V, 0, true>);
+    if (fk.mode == 1) return go(k_xfwd_w<LX, V, 1, true>);
+    if (fk.mode == 2) return go(k_xfwd_w<LX, V, 2, true>);
+    return go(k_xfwd_w<LX, V, 3, true>);
+}
+
+template <int LX>
+cudaError_t xinv(const Geom& g, int R, const float2* u, float2* y, const float2* x, const DevTarget& tg,
+                 const float2* beta, int beta_stride, bool tensor, const float2* tw, int* active,
+                 const FusedKrylov<float>& fk, cudaStream_t st) {
+    constexpr int V = kPlanInv<LX>;
+    using PL = XwPlan<LX, V>;
+    const size_t sm = xw_tile_bytes<PL>(xwi_rows<PL>());
+    const int nrows = tg.rows != nullptr ? tg.nrows : g.ny * g.nz;
+    dim3 grid((nrows + xwi_rows<PL>() - 1) / xwi_rows<PL>(), 3, R);
+    RowMap rm = row_map(g);
+    rm.pitch = g.ny * g.nz;
+    auto go = [&](auto kern) -> cudaError_t {
+        cudaError_t e = allow_smem(kern, sm);
+        if (e != cudaSuccess) return e;
+        PROF_BEGIN(st);
+        kern<<<grid, kXwiThreads, sm, st>>>(u, rm, y, x, tg.site_of, tg.comp_of, beta, beta_stride, tg.rows, nrows,
+                                            g.N, tw, active, fk.rhat, fk.st, fk.part, fk.cnt, fk.part_stride);
+        PROF_END(KK_XINV_C64, R, st);
+        return cudaGetLastError();
+    };
+    auto by_mode = [&](auto d) -> cudaError_t {
+        constexpr int D = decltype(d)::value;
+        const int mode = inverse_mode(fk.mode);
+        if (mode == 0) return go(k_xinv_w<LX, V, 0, D, true>);
+        if (mode == 1) return go(k_xinv_w<LX, V, 1, D, true>);
+        return go(k_xinv_w<LX, V, 2, D, true>);
+    };
+    cudaError_t e;
+    if (tensor) e = by_mode(std::integral_constant<int, kDiagTensor>{});
+    else if (tg.comp_of == nullptr) e = by_mode(std::integral_constant<int, kDiagSite>{});
+    else e = by_mode(std::integral_constant<int, kDiagComp>{});
+    if (e != cudaSuccess) return e;
+    return fused_finalize<float>(fk.mode, R, (int)(grid.x * grid.y), fk, active, st);
+}
+
+using SlabFn = cudaError_t (*)(const Geom&, int, float2*, const float4*, const Twiddles<float>&, const int*,
+                               cudaStream_t);
+SlabFn slab_fn(const Geom& g) {
+    switch (g.Ly) {
+        case 16: return slab_fn_16(g.Lz);
+        case 32: return slab_fn_32(g.Lz);
+        case 48: return slab_fn_48(g.Lz);
+        case 64: return slab_fn_64(g.Lz);
+        case 96: return slab_fn_96(g.Lz);
+        case 128: return slab_fn_128(g.Lz);
+        default: return nullptr;
+    }
+}
+
+}  // namespace
+
+bool slab_built(const Geom& g) { return slab_fn(g) != nullptr; }
+
+int64_t slab_green_size(const Geom& g) { return slab_green_all(g.hx(), g.Ly, g.Lz); }
+
+cudaError_t launch_slab_green(const Geom& g, const double2* gh64, float4* out, cudaStream_t st) {
+    auto go = [&](auto kern) {
+        kern<<<grid1d(slab_green_size(g), 256), 256, 0, st>>>(gh64, out, g.hx(), g.Ly);
+        return cudaGetLastError();
+    };
+    switch (g.Lz) {
+        case 16: return go(k_slab_green<16>);
+        case 32: return go(k_slab_green<32>);
+        case 48: return go(k_slab_green<48>);
+        case 64: return go(k_slab_green<64>);
+        case 96: return go(k_slab_green<96>);
+        case 128: return go(k_slab_green<128>);
+        default: return cudaErrorInvalidValue;
+    }
+}
+
+cudaError_t launch_slab_matvec(const Geom& g, int R, float2* x, float2* y, const PadWork<float>& w, const DevTarget& tg,
+                               const float2* beta, int beta_stride, const Twiddles<float>& tw, int* active,
+                               const FusedKrylov<float>& fk, cudaStream_t st) {
+    SlabFn slab = slab_fn(g);
+    if (slab == nullptr) return cudaErrorInvalidValue;
+    auto fwdx = [&]() -> cudaError_t { DDA_DISPATCH_L(g.Lx, xfwd, g, R, x, w.u2, tg, tw.x, active, fk, st); };
+    auto invx = [&]() -> cudaError_t {
+        DDA_DISPATCH_L(g.Lx, xinv, g, R, w.u2, y, x, tg, beta, beta_stride, w.beta_tensor, tw.x, active, fk, st);
+    };
+    cudaError_t e;
+    if ((e = fwdx()) != cudaSuccess) return e;
+    if ((e = slab(g, R, w.u2, w.slab, tw, active, st)) != cudaSuccess) return e;
+    return invx();
+}
+
+}  // namespace dda

@@ -151,7 +151,8 @@ template <class PL> __host__ __device__ constexpr int xwi_min_blocks() {
 }
 // the second BiCGstab scatter (MODE 2) keeps rhat and five sums besides: the
 // next larger budget (85 registers at 8 points per lane, 102 at 12)
-template <class PL, int MODE> __host__ __device__ constexpr int xwi_mode_min_blocks() {
+template <class PL, int MODE, bool TR> __host__ __device__ constexpr int xwi_mode_min_blocks() {
+    if (TR && PL::E > 16 && PL::E <= 24) return 4;
     return MODE != 2 ? xwi_min_blocks<PL>() : (PL::E <= 8 ? 6 : (PL::E <= 12 ? 5 : xwi_min_blocks<PL>()));
 }
 
@@ -171,11 +172,24 @@ template <int L> __device__ __forceinline__ const float2* stage_twiddles(float2*
     }
 }
 
+// ---- kx-major tiles ----------------------------------------------------------
+// The slab passes (slab.cuh) keep U kx-major, [R][3][LX][rows].  The x passes
+// then move a block's rows through shared memory as a tile [LX][SP], rows
+// fastest on the global side: SP spreads the 16 / NT pencils of a half-warp
+// (adjacent rows) and their lanes (adjacent x) over the banks.
+template <class PL> __host__ __device__ constexpr int xw_tile_stride(int rows) {
+    return rows + (PL::NT < 16 ? 16 / PL::NT : 1);
+}
+template <class PL> __host__ __device__ constexpr size_t xw_tile_bytes(int rows) {
+    const size_t tile = (size_t)PL::L * xw_tile_stride<PL>(rows), planes = (size_t)rows * xw_plane<PL>();
+    return (tile > planes ? tile : planes) * sizeof(float2);
+}
+
 // ---- x-forward: gather + row FFT, warp-local pencils -------------------------------
 // Same result as k_xfwd: rows (iy, iz) of the padded-to-LX/2 lattice, sites
 // x < LX/2 gathered through the lattice -> site map; MODE 1-3 form the
 // BiCGstab update in the gather and write it back (fused_gather).
-template <int LX, int V, int MODE>
+template <int LX, int V, int MODE, bool TR = false>
 __global__ void __launch_bounds__(kXwThreads, xwf_min_blocks<XwPlan<LX, V>>())
     k_xfwd_w(float2* __restrict__ X, float2* __restrict__ U, RowMap rm, const int* __restrict__ site_of, int nrows,
              int64_t N, const float2* __restrict__ tw, const int* __restrict__ active, FwdVecs<float2> fv) {
@@ -207,7 +221,8 @@ __global__ void __launch_bounds__(kXwThreads, xwf_min_blocks<XwPlan<LX, V>>())
     // does not wait for the slowest warp's gathers; in MODE 0 behind the
     // gathers themselves
     const C* tws = tw;
-    if constexpr (MODE != 0) tws = stage_twiddles<LX>(reinterpret_cast<C*>(smem_raw) + RPB * PS, tw);
+    constexpr int TWO = TR ? (int)(xw_tile_bytes<PL>(RPB) / sizeof(C)) : RPB * PS;
+    if constexpr (MODE != 0) tws = stage_twiddles<LX>(reinterpret_cast<C*>(smem_raw) + TWO, tw);
     C v[E];
     Gathered<C> gv[MODE == 3 ? NB0 * JN : 1];  // (MODE 3 keeps r and x for the stores)
 #pragma unroll
@@ -234,21 +249,35 @@ __global__ void __launch_bounds__(kXwThreads, xwf_min_blocks<XwPlan<LX, V>>())
                 fused_store<MODE>(xs, fv, off, s, o);
             }
     }
-    if constexpr (MODE == 0) tws = stage_twiddles<LX>(reinterpret_cast<C*>(smem_raw) + RPB * PS, tw);
+    if constexpr (MODE == 0) tws = stage_twiddles<LX>(reinterpret_cast<C*>(smem_raw) + TWO, tw);
     auto ld = [&](int pos) { return plane[pos]; };
     auto stf = [&](int pos, C val) { plane[pos] = val; };
     fft_stages<C, PL, -1, 0, decltype(ld), decltype(stf), true, XwExchange<PL>>(v, u, tws, ld, stf, true);
-    C* out = U + rm.at(r, c, ok ? row : 0, LX);
-    for_each_out<PL, -1, false>(u, [&](int idx, int pos) {
-        if (ok) out[pos] = v[idx];
-    });
+    if constexpr (TR) {
+        constexpr int SP = xw_tile_stride<PL>(RPB);
+        C* tile = reinterpret_cast<C*>(smem_raw);
+        __syncthreads();
+        for_each_out<PL, -1, false>(u, [&](int idx, int pos) { tile[pos * SP + p] = v[idx]; });
+        __syncthreads();
+        const int t = threadIdx.x % RPB, x0 = threadIdx.x / RPB, rt = blockIdx.x * RPB + t;
+        C* out = U + (((int64_t)r * 3 + c) * LX + x0) * rm.pitch + rt;
+        if (rt < nrows) {
+#pragma unroll
+            for (int i = 0; i < E; ++i) out[(int64_t)i * NT * rm.pitch] = tile[(x0 + i * NT) * SP + t];
+        }
+    } else {
+        C* out = U + rm.at(r, c, ok ? row : 0, LX);
+        for_each_out<PL, -1, false>(u, [&](int idx, int pos) {
+            if (ok) out[pos] = v[idx];
+        });
+    }
 }
 
 // ---- x-inverse: row IFFT + diagonal + scatter, warp-local pencils --------------
 // Same result as k_xinv (Y = conv + (1/alpha) X at the occupied sites, the
 // DIAG kinds, and the fused BiCGstab reductions of MODE 1 and 2).
-template <int LX, int V, int MODE, int DIAG>
-__global__ void __launch_bounds__(kXwiThreads, (xwi_mode_min_blocks<XwPlan<LX, V>, MODE>()))
+template <int LX, int V, int MODE, int DIAG, bool TR = false>
+__global__ void __launch_bounds__(kXwiThreads, (xwi_mode_min_blocks<XwPlan<LX, V>, MODE, TR>()))
     k_xinv_w(const float2* __restrict__ U, RowMap rm, float2* __restrict__ Y, const float2* __restrict__ X,
              const int* __restrict__ site_of, const uint8_t* __restrict__ comp_of, const float2* __restrict__ beta,
              int beta_stride, const int* __restrict__ rows, int nrows, int64_t N, const float2* __restrict__ tw,
@@ -274,15 +303,26 @@ __global__ void __launch_bounds__(kXwiThreads, (xwi_mode_min_blocks<XwPlan<LX, V
     C* ys = Y + off;
     constexpr bool TENSOR = DIAG == kDiagTensor;
     const C* br = beta + (int64_t)r * beta_stride + (TENSOR ? c * (beta_stride / 3) : 0);
-    const C* in = U + rm.at(r, c, ok ? row : 0, LX);
+    const C* in = U + (TR ? 0 : rm.at(r, c, ok ? row : 0, LX));
     // the row in the first stage's layout, then the site indices of the
     // lattice-half outputs and (up to 12 points per lane) the diagonal
     // operands: their latency is hidden by the transform
     C v[E];
+    C* tile = reinterpret_cast<C*>(smem_raw);
+    constexpr int SP = xw_tile_stride<PL>(RPB);
+    const int tt = threadIdx.x % RPB, x0 = threadIdx.x / RPB;  // TR: this thread's row of the tile, and its first x
+    if constexpr (TR) {
+        const int lt = blockIdx.x * RPB + tt;
+        const int rt = lt < nrows ? (rows != nullptr ? rows[lt] : lt) : -1;
+        const C* it = U + (((int64_t)r * 3 + c) * LX + x0) * rm.pitch + (rt < 0 ? 0 : rt);
 #pragma unroll
-    for (int q = 0; q < NB0; ++q)
+        for (int i = 0; i < E; ++i) v[i] = rt >= 0 ? it[(int64_t)i * NT * rm.pitch] : czero<C>();
+    } else {
 #pragma unroll
-        for (int j = 0; j < R0; ++j) v[q * R0 + j] = ok ? in[u + q * NT + j * (LX / R0)] : czero<C>();
+        for (int q = 0; q < NB0; ++q)
+#pragma unroll
+            for (int j = 0; j < R0; ++j) v[q * R0 + j] = ok ? in[u + q * NT + j * (LX / R0)] : czero<C>();
+    }
     int sidx[NO];
 #pragma unroll
     for (int q = 0; q < NBL; ++q)
@@ -308,7 +348,19 @@ __global__ void __launch_bounds__(kXwiThreads, (xwi_mode_min_blocks<XwPlan<LX, V
             }
         }
     };
+    if constexpr (TR) {
+#pragma unroll
+        for (int i = 0; i < E; ++i) tile[(x0 + i * NT) * SP + tt] = v[i];
+    }
     if constexpr (kHoist) load_operands();
+    if constexpr (TR) {
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < NB0; ++q)
+#pragma unroll
+            for (int j = 0; j < R0; ++j) v[q * R0 + j] = tile[(u + q * NT + j * (LX / R0)) * SP + p];
+        __syncthreads();
+    }
     auto ld = [&](int pos) { return plane[pos]; };
     auto stf = [&](int pos, C val) { plane[pos] = val; };
     fft_stages<C, PL, +1, 0, decltype(ld), decltype(stf), true, XwExchange<PL>>(v, u, tw, ld, stf, false);
