@@ -67,7 +67,7 @@ struct dda_ctx {
     bool has_target = false;
     int max_code = 0;
     DevTarget tg;
-    DevMem m_site_of, m_lat_of, m_comp_of, m_rows;
+    DevMem m_site_of, m_lat_of, m_comp_of, m_rows, m_row_start;
 
     // materials
     std::vector<cd> m;
@@ -1286,6 +1286,7 @@ dda_status dda_destroy(dda_ctx* ctx) {
     for (auto& m : ctx->pool) free_mem(m);
     free_mem(ctx->m_site_of);
     free_mem(ctx->m_rows);
+    free_mem(ctx->m_row_start);
     free_mem(ctx->m_lat_of);
     free_mem(ctx->m_comp_of);
     free_mem(ctx->m_gh64);
@@ -1347,17 +1348,20 @@ dda_status dda_set_target(dda_ctx* ctx, int nx, int ny, int nz, const uint8_t* c
             }
     if (lat_of.empty()) return ctx->fail(DDA_ERR_ARG, "target has no occupied site");
     g.N = (int64_t)lat_of.size();
-    // the x rows with at least one site (the x-inverse pass transforms only these)
-    std::vector<int> rows;
+    // the x rows with at least one site (the x-inverse pass transforms only
+    // these) and the first site of each
+    std::vector<int> rows, row_start;
     for (int iz = 0; iz < g.nz; ++iz)
         for (int iy = 0; iy < g.ny; ++iy) {
             const int64_t r0 = ((int64_t)iz * g.ny + iy) * g.nx;
             for (int ix = 0; ix < g.nx; ++ix)
                 if (site_of[r0 + ix] >= 0) {
                     rows.push_back(iz * g.ny + iy);
+                    row_start.push_back(site_of[r0 + ix]);
                     break;
                 }
         }
+    row_start.push_back((int)g.N);
     cudaSetDevice(ctx->device);
     ctx->prepared = false;
     ctx->has32 = false;
@@ -1370,11 +1374,14 @@ dda_status dda_set_target(dda_ctx* ctx, int nx, int ny, int nz, const uint8_t* c
     CU(cudaMemcpy(ctx->m_comp_of.p, comp_of.data(), g.N, cudaMemcpyHostToDevice));
     if ((s = ensure(ctx, ctx->m_rows, rows.size() * sizeof(int))) != DDA_OK) return s;
     CU(cudaMemcpy(ctx->m_rows.p, rows.data(), rows.size() * sizeof(int), cudaMemcpyHostToDevice));
+    if ((s = ensure(ctx, ctx->m_row_start, row_start.size() * sizeof(int))) != DDA_OK) return s;
+    CU(cudaMemcpy(ctx->m_row_start.p, row_start.data(), row_start.size() * sizeof(int), cudaMemcpyHostToDevice));
     ctx->tg.site_of = (int*)ctx->m_site_of.p;
     ctx->tg.lat_of = (int*)ctx->m_lat_of.p;
     ctx->tg.comp_of = (uint8_t*)ctx->m_comp_of.p;
     ctx->tg.rows = (const int*)ctx->m_rows.p;
     ctx->tg.nrows = (int)rows.size();
+    ctx->tg.row_start = (const int*)ctx->m_row_start.p;
     ctx->g = g;
     ctx->zsched.clear();
     ctx->max_code = maxc;
@@ -1964,44 +1971,44 @@ dda_status farfield_run(dda_ctx* ctx, int R, const std::vector<double>& khat, co
     const Geom& g = ctx->g;
     const int64_t N = g.N;
     if (g.ox > 1024 || g.oy > 1024 || g.oz > 1024) return ctx->fail(DDA_ERR_SIZE, "far field: lattice above 1024");
-    const int Lm = std::max(g.ox, std::max(g.oy, g.oz)), tab_len = 3 * Lm;
-    const double kd = ctx->kd, c[3] = {0.5 * (g.ox - 1), 0.5 * (g.oy - 1), 0.5 * (g.oz - 1)};
-    std::vector<double> dirs((size_t)R * ndir * 3);
-    for (int r = 0; r < R; ++r) {
+    const double kd = ctx->kd;
+    // the two polarizations of a direction share its Lab Frame, and with it all
+    // their scattering directions
+    bool pairs = R % 2 == 0;
+    for (int r = 0; r < R && pairs; r += 2) pairs = std::memcmp(&khat[3 * r], &khat[3 * r + 3], 3 * sizeof(double)) == 0;
+    const int NR = pairs ? 2 : 1, groups = R / NR;
+    std::vector<double> dirs((size_t)groups * ndir * 3);
+    std::vector<double> ctp(4 * (size_t)ndir);  // cos, sin of theta and phi
+    for (int d = 0; d < ndir; ++d) {
+        ctp[4 * d] = std::cos(theta[d]);
+        ctp[4 * d + 1] = std::sin(theta[d]);
+        ctp[4 * d + 2] = std::cos(phi[d]);
+        ctp[4 * d + 3] = std::sin(phi[d]);
+    }
+    for (int r = 0; r < groups; ++r) {
         double xl[3], yl[3], zl[3];
-        lab_frame(&khat[3 * r], xl, yl, zl);
+        lab_frame(&khat[3 * r * NR], xl, yl, zl);
         for (int d = 0; d < ndir; ++d) {
-            const double ct = std::cos(theta[d]), st = std::sin(theta[d]), cp = std::cos(phi[d]), sp = std::sin(phi[d]);
+            const double ct = ctp[4 * d], st = ctp[4 * d + 1], cp = ctp[4 * d + 2], sp = ctp[4 * d + 3];
             double* n = &dirs[((size_t)r * ndir + d) * 3];
             for (int a = 0; a < 3; ++a) n[a] = ct * xl[a] + st * cp * yl[a] + st * sp * zl[a];
         }
     }
-    const size_t ntab = (size_t)R * ndir * tab_len;
-    std::vector<int> lat(N);
-    std::vector<unsigned> xyz(N);
-    CU(cudaMemcpy(lat.data(), ctx->tg.lat_of, N * sizeof(int), cudaMemcpyDeviceToHost));
-    for (int64_t j = 0; j < N; ++j) {
-        const int l = lat[j];
-        const unsigned ix = l % g.nx, iy = (l / g.nx) % g.ny, iz = l / (g.nx * g.ny);
-        xyz[j] = ix | (iy << 10) | (iz << 20);
-    }
+    FarGeom f{g.ox, g.oy, g.oz, ndir, far_padded(ndir)};
+    const size_t ntab = (size_t)groups * f.Lt() * f.ndp;
     NearWork w;
     cudaError_t ce = cudaSuccess;
     auto alloc = [&](size_t bytes) { return ce == cudaSuccess ? w.get(bytes, ce) : nullptr; };
-    unsigned* d_xyz = (unsigned*)alloc(N * sizeof(unsigned));
-    double2* d_P64 = (double2*)alloc((size_t)R * 3 * N * sizeof(double2));
-    C* d_P = sizeof(T) == 8 ? (C*)d_P64 : (C*)alloc((size_t)R * 3 * N * sizeof(C));
+    double2* d_P = (double2*)alloc((size_t)R * 3 * N * sizeof(double2));
     C* d_tabs = (C*)alloc(ntab * sizeof(C));
     double* d_dirs = (double*)alloc(dirs.size() * sizeof(double));
     double2* d_F = (double2*)alloc((size_t)R * ndir * 3 * sizeof(double2));
     if (ce != cudaSuccess) return ctx->cuda_fail(ce, "far-field workspace");
     cudaStream_t st = ctx->stream;
-    CU(cudaMemcpyAsync(d_xyz, xyz.data(), N * sizeof(unsigned), cudaMemcpyHostToDevice, st));
-    CU(cudaMemcpyAsync(d_P64, P_host, (size_t)R * 3 * N * sizeof(double2), cudaMemcpyHostToDevice, st));
-    if (sizeof(T) != 8) CU(launch_c128_to_c64v((int64_t)R * 3 * N, d_P64, (float2*)d_P, st));
     CU(cudaMemcpyAsync(d_dirs, dirs.data(), dirs.size() * sizeof(double), cudaMemcpyHostToDevice, st));
-    CU(launch_phase_tables<C>((int64_t)R * ndir, Lm, c, kd, d_dirs, d_tabs, st));
-    CU(launch_farfield<C>(R, N, d_xyz, d_P, ndir, tab_len, d_tabs, d_dirs, kd, d_F, st));
+    CU(launch_phase_tables<C>(f, groups, kd, d_dirs, d_tabs, st));
+    CU(cudaMemcpyAsync(d_P, P_host, (size_t)R * 3 * N * sizeof(double2), cudaMemcpyHostToDevice, st));
+    CU(launch_farfield<C>(g, ctx->tg, f, groups, NR, d_P, d_tabs, d_dirs, kd, d_F, st));
     F.resize((size_t)R * ndir * 3);
     CU(cudaMemcpyAsync(F.data(), d_F, F.size() * sizeof(double2), cudaMemcpyDeviceToHost, st));
     CU(sync_collect(ctx));

@@ -43,6 +43,7 @@ struct DevTarget {
     // (a row without sites has no output); null: every row
     const int* rows = nullptr;
     int nrows = 0;
+    const int* row_start = nullptr;  // [nrows + 1] first site of each (the far field's sums)
 };
 
 // Twiddle tables, one per padded axis: exp(-2 pi i m/L), m < L.
