@@ -1519,7 +1519,7 @@ dda_status dda_prepare(dda_ctx* ctx, double lambda_vac, double aeff, dda_precisi
     const int64_t oct = 6 * g.oct_per_comp();
     if ((s = ensure(ctx, ctx->m_gh64, oct * sizeof(double2))) != DDA_OK) return s;
     DevMem scratch;
-    const size_t sb = (size_t)6 * g.Lx * g.Ly * g.Lz * sizeof(double2);
+    const size_t sb = (size_t)green_scratch_size(g) * sizeof(double2);
     cudaError_t e = cudaMalloc(&scratch.p, sb);
     if (e != cudaSuccess) return ctx->cuda_fail(e, "cudaMalloc(Green tensor scratch)");
     e = launch_green_fft(g, ctx->kd, (double2*)scratch.p, (double2*)ctx->m_gh64.p, tw_of<double>(ctx), ctx->stream);
@@ -1827,7 +1827,7 @@ dda_status nearfield_run(dda_ctx* ctx, int R, const double* P_host, const int di
     }
     {
         DevMem scratch;
-        CU(cudaMalloc(&scratch.p, (size_t)6 * g.Lx * g.Ly * g.Lz * sizeof(double2)));
+        CU(cudaMalloc(&scratch.p, (size_t)green_scratch_size(g) * sizeof(double2)));
         Twiddles<double> t{tw64[0], tw64[1], tw64[2]};
         cudaError_t e1 = launch_green_fft(g, ctx->kd, (double2*)scratch.p, gh64, t, st);
         if (e1 == cudaSuccess) e1 = cudaStreamSynchronize(st);

@@ -179,7 +179,8 @@ cudaError_t launch_matvec(const Geom& g, int R, const cx<T>* x, cx<T>* y, const 
                           const Twiddles<T>& tw, const int* active, cudaStream_t st);
 
 // Build the octant of FFT(g)/(Lx Ly Lz) of the six Green-tensor components
-// (xx, xy, xz, yy, yz, zz) in FP64.  scratch: 6*Lx*Ly*Lz double2.
+// (xx, xy, xz, yy, yz, zz) in FP64.  scratch: green_scratch_size double2.
+int64_t green_scratch_size(const Geom& g);
 cudaError_t launch_green_fft(const Geom& g, double kd, double2* scratch, double2* ghat64,
                              const Twiddles<double>& tw, cudaStream_t st);
 

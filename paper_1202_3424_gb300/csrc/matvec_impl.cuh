@@ -287,10 +287,10 @@ __global__ void __launch_bounds__(tp_x<LX, sizeof(cx<T>)>() * XPlan<LX, sizeof(c
     if constexpr (MODE != 0) fused_partials<C, MODE>(d, part, r, part_stride);
 }
 
-// ---- strided pencils (y passes; y and z passes of the Green tensor) -----------
+// ---- strided pencils (y passes) -----------
 // Pencil (b, w): points at src + b*src_bstride + w + pos*pt_stride; outputs
 // to dst likewise.  MODE 0: forward with input positions >= L/2 zero;
-// MODE 1: inverse keeping positions < L/2; MODE 2: full forward transform.
+// MODE 1: inverse keeping positions < L/2.
 // TP pencils adjacent in w per block, so loads and stores coalesce across w.
 // Radix plan variant V = 1 (complex64 y passes, tuned like the other passes):
 // 128 = 8 x 16, 192 = 8 x 8 x 3, 256 = 16 x 16, 512 = 32 x 16, one exchange
@@ -785,39 +785,6 @@ __global__ void __launch_bounds__(zreg_threads<ZrPlan<LZ, V>>(), zreg_min_blocks
     }
 }
 
-// In-place forward FFT of dense rows of length LX (Green tensor x pass).
-template <int LX>
-__global__ void __launch_bounds__(tp_x<LX, 16>() * Plan<LX>::NT)
-    k_xfull(double2* __restrict__ data, int64_t nrows, const double2* __restrict__ tw) {
-    using C = double2;
-    using PL = Plan<LX>;
-    constexpr int TP = tp_x<LX, 16>(), SP = TP + 1;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    C* buf = reinterpret_cast<C*>(smem_raw);
-    const int64_t row0 = (int64_t)blockIdx.x * TP;
-    for (int e = threadIdx.x; e < TP * LX; e += blockDim.x) {
-        const int t2 = e / LX, x = e - t2 * LX;
-        const int64_t row = row0 + t2;
-        buf[x * SP + t2] = row < nrows ? data[row * LX + x] : czero<C>();
-    }
-    __syncthreads();
-    const int t = threadIdx.x % TP, u = threadIdx.x / TP;
-    C* bt = buf + t;
-    C v[PL::E];
-    auto first = [&](int pos) { return bt[pos * SP]; };
-    auto ld = [&](int pos) { return bt[pos * SP]; };
-    auto st = [&](int pos, C val) { bt[pos * SP] = val; };
-    pencil_fft<C, PL, -1, false>(v, u, tw, first, ld, st);
-    __syncthreads();
-    for_each_out<PL, -1, false>(u, [&](int idx, int pos) { bt[pos * SP] = v[idx]; });
-    __syncthreads();
-    for (int e = threadIdx.x; e < TP * LX; e += blockDim.x) {
-        const int t2 = e / LX, x = e - t2 * LX;
-        const int64_t row = row0 + t2;
-        if (row < nrows) data[row * LX + x] = buf[x * SP + t2];
-    }
-}
-
 // ---- host launchers -------------------------------------------------------------
 // Give a kernel the maximum shared-memory carveout and, above 48 KB, the
 // dynamic shared-memory size it needs -- once per kernel
@@ -1082,9 +1049,7 @@ template <typename T> struct LaunchX {
         }
         if (mode == 0)
             return strided_mode<0, L>(src, dst, pt_stride, width, sb, db, batches, per_rhs, tw, active, st, kind, units);
-        if (mode == 1)
-            return strided_mode<1, L>(src, dst, pt_stride, width, sb, db, batches, per_rhs, tw, active, st, kind, units);
-        return strided_mode<2, L>(src, dst, pt_stride, width, sb, db, batches, per_rhs, tw, active, st, kind, units);
+        return strided_mode<1, L>(src, dst, pt_stride, width, sb, db, batches, per_rhs, tw, active, st, kind, units);
     }
     template <int LZ>
     static cudaError_t zconv(const Geom& g, int R, cx<T>* u2, const cx<T>* gh, const cx<T>* tw, const int* active,
