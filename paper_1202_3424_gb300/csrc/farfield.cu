@@ -49,9 +49,12 @@ template <int n, typename C> __device__ __forceinline__ void read_words(C (&v)[n
 // warps, on rows of their own, share.  Both polarizations of a direction (NR
 // = 2) share it too: per site and lane 12 TD NR multiply-adds for TD table
 // words.  Bound by the FP32 pipes; 16 RHS x 2172 directions x 102984 sites:
-// 5.60 -> 2.30 ms.
+// 5.60 -> 2.30 ms with two directions a lane, 2.1 ms with four (at two thirds of
+// the issue slots: multiply-adds of three different registers run at 87 of 128
+// lanes).  In packed pairs, which need P's parts twice in shared memory, it took
+// 2.6 ms.
 template <typename C, int NR, int TD>
-__global__ void __launch_bounds__(kFFWarps * 32)
+__global__ void __launch_bounds__(kFFWarps * 32, 2)
     k_farfield(const double2* __restrict__ P, int64_t N, const int* __restrict__ rows,
                const int* __restrict__ row_start, int nrows, int per_chunk, const int* __restrict__ lat_of, int nxe,
                int nye, FarGeom f, const C* __restrict__ tabs, const double* __restrict__ dirs, double kd,
@@ -68,7 +71,10 @@ __global__ void __launch_bounds__(kFFWarps * 32)
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     C* wb = buf + warp * 32 * NC;
     int* wi = bix + warp * 32;
-    const C* tl = tab + lane * TD;
+    // direction t of a lane: neighbouring pairs, one 16-byte word apart from the
+    // next lane's, the second pair of four 64 directions on
+    auto dir = [&](int t) { return TD == 4 ? t / 2 * 64 + lane * 2 + t % 2 : lane * TD + t; };
+    const C* tl = tab + dir(0);
     const double2* Pg = P + (int64_t)grp * NC * N;
     C tot[TD][NC];
 #pragma unroll
@@ -96,7 +102,12 @@ __global__ void __launch_bounds__(kFFWarps * 32)
             for (int i = 0; i < m; ++i) {
                 const C* ex = tl + wi[i];
                 C e[TD], p[NC];
-                read_words(e, ex);
+                if constexpr (TD == 4) {
+                    read_words(reinterpret_cast<C(&)[2]>(e[0]), ex);
+                    read_words(reinterpret_cast<C(&)[2]>(e[2]), ex + 64);
+                } else {
+                    read_words(e, ex);
+                }
                 read_words(p, wb + i * NC);
 #pragma unroll
                 for (int t = 0; t < TD; ++t)
@@ -111,7 +122,7 @@ __global__ void __launch_bounds__(kFFWarps * 32)
         }
 #pragma unroll
         for (int t = 0; t < TD; ++t) {
-            const int d = lane * TD + t;
+            const int d = dir(t);
             const C ph = cmul(gt[(int64_t)(f.nx + iy) * f.ndp + d], gt[(int64_t)(f.nx + f.ny + iz) * f.ndp + d]);
 #pragma unroll
             for (int c = 0; c < NC; ++c) tot[t][c] = cadd(tot[t][c], cmul(acc[t][c], ph));
@@ -122,7 +133,7 @@ __global__ void __launch_bounds__(kFFWarps * 32)
 #pragma unroll
     for (int t = 0; t < TD; ++t)
 #pragma unroll
-        for (int c = 0; c < NC; ++c) red[(warp * NC + c) * ND + lane * TD + t] = tot[t][c];
+        for (int c = 0; c < NC; ++c) red[(warp * NC + c) * ND + dir(t)] = tot[t][c];
     __syncthreads();
     for (int e = threadIdx.x; e < ND * NR; e += kFFWarps * 32) {
         const int r = e / ND, td = e % ND, d = d0 + td;
@@ -193,10 +204,17 @@ cudaError_t launch_farfield(const Geom& g, const DevTarget& tg, const FarGeom& f
                             const C* tabs, const double* dirs, double kd, double2* F, cudaStream_t st) {
     cudaError_t e = cudaMemsetAsync(F, 0, (size_t)groups * NR * f.ndir * 3 * sizeof(double2), st);
     if (e != cudaSuccess) return e;
-    // directions per lane: two, or one in FP64 (whose table words are twice as wide)
-    constexpr int TD = sizeof(C) == 8 ? 2 : 1, ND = 32 * TD;
-    const size_t work = (size_t)f.nx * ND * sizeof(C) + (size_t)kFFWarps * 32 * (NR * 3 * sizeof(C) + sizeof(int));
-    const size_t sm = std::max(work, (size_t)kFFWarps * NR * 3 * ND * sizeof(C));
+    // directions per lane: four while two blocks' tables fit an SM, else two; one
+    // in FP64 (whose table words are twice as wide)
+    constexpr int TW = sizeof(C) == 8 ? 4 : 1, TN = sizeof(C) == 8 ? 2 : 1;
+    auto smem = [&](int td) {
+        const size_t work =
+            (size_t)f.nx * 32 * td * sizeof(C) + (size_t)kFFWarps * 32 * (NR * 3 * sizeof(C) + sizeof(int));
+        return std::max(work, (size_t)kFFWarps * NR * 3 * 32 * td * sizeof(C));
+    };
+    const bool wide = TW > TN && smem(TW) <= 112 * 1024;
+    const int ND = 32 * (wide ? TW : TN);
+    const size_t sm = smem(wide ? TW : TN);
     // row chunks: at most kFFRows rows, and enough blocks for two waves of the 152 SMs
     const int tiles = (f.ndir + ND - 1) / ND;
     const int64_t want = (4 * 152 + (int64_t)tiles * groups - 1) / ((int64_t)tiles * groups);
@@ -215,7 +233,8 @@ cudaError_t launch_farfield(const Geom& g, const DevTarget& tg, const FarGeom& f
         PROF_END(KK_FARFIELD, groups * NR, st);
         return cudaGetLastError();
     };
-    return NR == 2 ? go(k_farfield<C, 2, TD>) : go(k_farfield<C, 1, TD>);
+    if (wide) return NR == 2 ? go(k_farfield<C, 2, TW>) : go(k_farfield<C, 1, TW>);
+    return NR == 2 ? go(k_farfield<C, 2, TN>) : go(k_farfield<C, 1, TN>);
 }
 
 template cudaError_t launch_farfield<float2>(const Geom&, const DevTarget&, const FarGeom&, int, int, const double2*,

@@ -18,7 +18,7 @@ struct FarGeom {
     int ndir, ndp;
     int Lt() const { return nx + ny + nz; }
 };
-inline int far_padded(int ndir) { return (ndir + 63) / 64 * 64; }
+inline int far_padded(int ndir) { return (ndir + 127) / 128 * 128; }
 
 // dirs[(group*ndir + d)*3 + a]: the unit vectors.  C = float2 or double2.
 template <typename C>
