@@ -4,6 +4,8 @@
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_runtime.h>
+#include <sys/mman.h>
+#include <unistd.h>
 
 #include <algorithm>
 #include <array>
@@ -15,6 +17,7 @@
 #include <map>
 #include <mutex>
 #include <string>
+#include <thread>
 #include <vector>
 
 #include "dda.h"
@@ -35,6 +38,7 @@ constexpr double kB1 = -1.8915316, kB2 = 0.1648469, kB3 = -1.7700004;
 struct DevMem {
     void* p = nullptr;
     size_t bytes = 0;
+    bool view = false;  // part of another buffer: not owned
 };
 
 // Inner-solve vectors.  BiCGstab: b, x, r, rhat, p, v, s, t.  BiCGstab(2)
@@ -107,6 +111,13 @@ struct dda_ctx {
     // per SM), so they are opt-in.
     int force_slices = 0;
     int* h_count = nullptr;  // pinned
+    // pinned staging of the small tables that go to and from the device, one
+    // copy per call in place of one per table (grown on demand, at most
+    // kStageMax); stage_ev marks the last copy out of it
+    char* h_stage = nullptr;
+    size_t h_stage_bytes = 0;
+    cudaEvent_t stage_ev = nullptr;
+    int tw_len[3] = {0, 0, 0};  // lengths the twiddle tables hold
     Profiler prof;
 
     dda_status fail(dda_status code, const char* fmt, ...) {
@@ -155,6 +166,10 @@ enum Slot {
     S_BETA64, S_BETA32, S_W, S_KHAT, S_EPOL,
     S_MV_X32, S_MV_Y32, S_GRAD, S_DBETA,
     S_BETADF, S_XDF, S_YDF, S_TUNE, S_IN_U2,
+    S_TABLES,  // holds S_BETA64, S_BETA32, S_BETADF, S_W, S_KHAT, S_EPOL
+    S_SCALARS, // holds S_STATE, S_NORM_B, S_NORM_R, S_QSUM, S_TOLREL, S_SCALE, S_COEF, S_OUTER
+    S_GREEN,   // scratch of dda_prepare's transforms
+    S_FIELD,   // workspace of the near and far field calls
     S_NSLOTS
 };
 
@@ -179,14 +194,103 @@ dda_status ensure(dda_ctx* ctx, DevMem& m, size_t bytes, bool zero = false) {
     return DDA_OK;
 }
 
+// Scratch that no captured graph refers to.
+dda_status ensure_scratch(dda_ctx* ctx, DevMem& m, size_t bytes) {
+    if (m.bytes >= bytes && m.p != nullptr) return DDA_OK;
+    if (m.p) cudaFree(m.p);
+    m = DevMem{};
+    CU(cudaMalloc(&m.p, bytes < 256 ? 256 : bytes));
+    m.bytes = bytes < 256 ? 256 : bytes;
+    return DDA_OK;
+}
+
 template <typename P> P* slot(dda_ctx* ctx, int s) { return reinterpret_cast<P*>(ctx->pool[s].p); }
 
 size_t align256(size_t b) { return (b + 255) & ~size_t(255); }
 
 void free_mem(DevMem& m) {
-    if (m.p) cudaFree(m.p);
-    m.p = nullptr;
-    m.bytes = 0;
+    if (m.p && !m.view) cudaFree(m.p);
+    m = DevMem{};
+}
+
+// Scratch that a call keeps for the next one only up to this size.
+constexpr size_t kKeepMax = (size_t)1 << 30;
+constexpr size_t kStageMax = (size_t)4 << 20;
+
+// Consecutive 256-byte-aligned parts of one buffer, laid out the same in the
+// staging area and on the device.
+struct Parts {
+    size_t total = 0;
+    size_t add(size_t bytes) {
+        const size_t at = total;
+        total += align256(bytes);
+        return at;
+    }
+};
+// The staging area with room for `bytes`, its last copy finished; null if they
+// are too many for it.
+dda_status stage(dda_ctx* ctx, size_t bytes, char** out) {
+    *out = nullptr;
+    if (bytes > kStageMax) return DDA_OK;
+    if (ctx->stage_ev == nullptr) {
+        CU(cudaEventCreateWithFlags(&ctx->stage_ev, cudaEventDisableTiming));
+    } else if (cudaEventSynchronize(ctx->stage_ev) != cudaSuccess) {
+        // (a call inside a stream capture, which fails, leaves an event that cannot be waited for)
+        cudaGetLastError();
+        cudaEventDestroy(ctx->stage_ev);
+        ctx->stage_ev = nullptr;
+        CU(cudaStreamSynchronize(ctx->stream));
+        CU(cudaEventCreateWithFlags(&ctx->stage_ev, cudaEventDisableTiming));
+    }
+    if (bytes > ctx->h_stage_bytes) {
+        if (ctx->h_stage) cudaFreeHost(ctx->h_stage);
+        ctx->h_stage = nullptr;
+        ctx->h_stage_bytes = 0;
+        CU(cudaMallocHost(&ctx->h_stage, std::max(bytes, (size_t)64 << 10)));
+        ctx->h_stage_bytes = std::max(bytes, (size_t)64 << 10);
+    }
+    *out = ctx->h_stage;
+    return DDA_OK;
+}
+// Page in a large host buffer that the device is about to fill, on two threads
+// (a copy into fresh memory runs at the rate of one core's page faults: 85 MB
+// 3.7 ms, against 0.5 ms once paged in).  MADV_POPULATE_WRITE leaves the
+// contents alone; writing each page's own bytes back instead would map the zero
+// page first, and replacing that stalls on the device's mappings (70 ms).
+// wait() before the copy; the destructor waits too.
+class PageIn {
+    std::vector<std::thread> threads_;
+
+  public:
+    void start(void* p, size_t bytes) {
+#ifdef MADV_POPULATE_WRITE
+        constexpr size_t kMin = (size_t)8 << 20, kThreads = 2;
+        if (p == nullptr || bytes < kMin) return;
+        const size_t page = (size_t)sysconf(_SC_PAGESIZE);
+        const uintptr_t lo = ((uintptr_t)p + page - 1) / page * page, hi = ((uintptr_t)p + bytes) / page * page;
+        const size_t per = ((hi - lo) / kThreads + page) / page * page;
+        try {
+            for (uintptr_t at = lo; at < hi; at += per)
+                threads_.emplace_back([at, len = std::min<size_t>(per, hi - at)] {
+                    madvise((void*)at, len, MADV_POPULATE_WRITE);
+                });
+        } catch (...) {
+            // no thread to be had: the copy pages the rest in
+        }
+#endif
+    }
+    void wait() {
+        for (auto& t : threads_) t.join();
+        threads_.clear();
+    }
+    ~PageIn() { wait(); }
+};
+
+void set_view(dda_ctx* ctx, int slot, int owner, size_t at, size_t bytes) {
+    DevMem& m = ctx->pool[slot];
+    m.p = static_cast<char*>(ctx->pool[owner].p) + at;
+    m.bytes = bytes;
+    m.view = true;
 }
 
 // S = sum_a khat_a^2 |e_a|^2 for a unit e: for a real e this is Draine &
@@ -317,30 +421,39 @@ dda_status upload_tables(dda_ctx* ctx, int R, const std::vector<double>& k, cons
     std::vector<double> w;
     dda_status s;
     if ((s = diag_tables(ctx, R, k, e, b, &w)) != DDA_OK) return s;
-    std::vector<double2> b64(b.size());
-    std::vector<float2> b32(b.size());
-    std::vector<cdfl> bdf(b.size());
-    for (size_t i = 0; i < b.size(); ++i) {
-        b64[i] = make_double2(b[i].real(), b[i].imag());
-        b32[i] = make_float2((float)b[i].real(), (float)b[i].imag());
-        bdf[i] = cdfl{dfl(b[i].real()), dfl(b[i].imag())};
+    const size_t nb = b.size();
+    Parts parts;
+    const size_t o64 = parts.add(nb * sizeof(double2)), o32 = parts.add(nb * sizeof(float2)),
+                 odf = parts.add(nb * sizeof(cdfl)), ow = parts.add(w.size() * sizeof(double)),
+                 ok = parts.add(k.size() * sizeof(double)), oe = parts.add(3 * (size_t)R * sizeof(double2));
+    if ((s = ensure(ctx, ctx->pool[S_TABLES], parts.total)) != DDA_OK) return s;
+    set_view(ctx, S_BETA64, S_TABLES, o64, nb * sizeof(double2));
+    set_view(ctx, S_BETA32, S_TABLES, o32, nb * sizeof(float2));
+    set_view(ctx, S_BETADF, S_TABLES, odf, nb * sizeof(cdfl));
+    set_view(ctx, S_W, S_TABLES, ow, w.size() * sizeof(double));
+    set_view(ctx, S_KHAT, S_TABLES, ok, k.size() * sizeof(double));
+    set_view(ctx, S_EPOL, S_TABLES, oe, 3 * (size_t)R * sizeof(double2));
+    // through the staging area (the caller's own synchronization ends the copy),
+    // or, for tables of many sites, from a buffer of this call
+    char* h = nullptr;
+    if ((s = stage(ctx, parts.total, &h)) != DDA_OK) return s;
+    std::vector<char> own;
+    if (h == nullptr) {
+        own.resize(parts.total);
+        h = own.data();
     }
-    if ((s = ensure(ctx, ctx->pool[S_BETA64], b64.size() * sizeof(double2))) != DDA_OK) return s;
-    if ((s = ensure(ctx, ctx->pool[S_BETA32], b32.size() * sizeof(float2))) != DDA_OK) return s;
-    if ((s = ensure(ctx, ctx->pool[S_W], w.size() * sizeof(double))) != DDA_OK) return s;
-    CU(cudaMemcpyAsync(ctx->pool[S_BETA64].p, b64.data(), b64.size() * sizeof(double2), cudaMemcpyHostToDevice, ctx->stream));
-    CU(cudaMemcpyAsync(ctx->pool[S_BETA32].p, b32.data(), b32.size() * sizeof(float2), cudaMemcpyHostToDevice, ctx->stream));
-    if ((s = ensure(ctx, ctx->pool[S_BETADF], bdf.size() * sizeof(cdfl))) != DDA_OK) return s;
-    CU(cudaMemcpyAsync(ctx->pool[S_BETADF].p, bdf.data(), bdf.size() * sizeof(cdfl), cudaMemcpyHostToDevice, ctx->stream));
-    CU(cudaMemcpyAsync(ctx->pool[S_W].p, w.data(), w.size() * sizeof(double), cudaMemcpyHostToDevice, ctx->stream));
-    std::vector<double2> e2(3 * (size_t)R);
-    for (size_t i = 0; i < e2.size(); ++i) e2[i] = make_double2(e[i].real(), e[i].imag());
-    if ((s = ensure(ctx, ctx->pool[S_KHAT], k.size() * sizeof(double))) != DDA_OK) return s;
-    if ((s = ensure(ctx, ctx->pool[S_EPOL], e2.size() * sizeof(double2))) != DDA_OK) return s;
-    CU(cudaMemcpyAsync(ctx->pool[S_KHAT].p, k.data(), k.size() * sizeof(double), cudaMemcpyHostToDevice, ctx->stream));
-    CU(cudaMemcpyAsync(ctx->pool[S_EPOL].p, e2.data(), e2.size() * sizeof(double2), cudaMemcpyHostToDevice, ctx->stream));
-    // the host vectors go out of scope: finish the copies first
-    CU(sync_collect(ctx));
+    for (size_t i = 0; i < nb; ++i) {
+        reinterpret_cast<double2*>(h + o64)[i] = make_double2(b[i].real(), b[i].imag());
+        reinterpret_cast<float2*>(h + o32)[i] = make_float2((float)b[i].real(), (float)b[i].imag());
+        reinterpret_cast<cdfl*>(h + odf)[i] = cdfl{dfl(b[i].real()), dfl(b[i].imag())};
+    }
+    std::memcpy(h + ow, w.data(), w.size() * sizeof(double));
+    std::memcpy(h + ok, k.data(), k.size() * sizeof(double));
+    for (size_t i = 0; i < 3 * (size_t)R; ++i)
+        reinterpret_cast<double2*>(h + oe)[i] = make_double2(e[i].real(), e[i].imag());
+    CU(cudaMemcpyAsync(ctx->pool[S_TABLES].p, h, parts.total, cudaMemcpyHostToDevice, ctx->stream));
+    if (own.empty()) CU(cudaEventRecord(ctx->stage_ev, ctx->stream));
+    else CU(sync_collect(ctx));  // the buffer goes out of scope
     return DDA_OK;
 }
 
@@ -848,6 +961,23 @@ struct RhsTrack {
     bool done = false;
 };
 
+// The per-RHS scalars of a solve, one part of S_SCALARS after another, ordered
+// so that each direction is one copy: the norms and the state come back, the
+// state and what follows it go down.
+struct ScalarParts {
+    Parts p;
+    size_t norm_b, norm_r, state, tolrel, scale, coef, outer;
+    explicit ScalarParts(int R) {
+        norm_b = p.add(R * sizeof(double));
+        norm_r = p.add(R * sizeof(double));
+        state = p.add(R * sizeof(KState));
+        tolrel = p.add(R * sizeof(double));
+        scale = p.add(R * sizeof(double));
+        coef = p.add(R * sizeof(double));
+        outer = p.add(R * sizeof(int));
+    }
+};
+
 dda_status ensure_common(dda_ctx* ctx, int R) {
     dda_status s;
     const size_t nb = (size_t)R * partial_stride(ctx) * sizeof(double2);
@@ -855,11 +985,17 @@ dda_status ensure_common(dda_ctx* ctx, int R) {
     if (ctx->pool[S_CNT].bytes < R * sizeof(unsigned)) {
         if ((s = ensure(ctx, ctx->pool[S_CNT], R * sizeof(unsigned), true)) != DDA_OK) return s;
     }
-    for (int sl : {S_ACTIVE, S_WANT, S_OUTER})
+    for (int sl : {S_ACTIVE, S_WANT})
         if ((s = ensure(ctx, ctx->pool[sl], R * sizeof(int))) != DDA_OK) return s;
-    for (int sl : {S_TOLREL, S_SCALE, S_COEF, S_NORM_B, S_NORM_R})
-        if ((s = ensure(ctx, ctx->pool[sl], R * sizeof(double))) != DDA_OK) return s;
-    if ((s = ensure(ctx, ctx->pool[S_STATE], R * sizeof(KState))) != DDA_OK) return s;
+    const ScalarParts sp(R);
+    if ((s = ensure(ctx, ctx->pool[S_SCALARS], sp.p.total)) != DDA_OK) return s;
+    set_view(ctx, S_NORM_B, S_SCALARS, sp.norm_b, R * sizeof(double));
+    set_view(ctx, S_NORM_R, S_SCALARS, sp.norm_r, R * sizeof(double));
+    set_view(ctx, S_STATE, S_SCALARS, sp.state, R * sizeof(KState));
+    set_view(ctx, S_TOLREL, S_SCALARS, sp.tolrel, R * sizeof(double));
+    set_view(ctx, S_SCALE, S_SCALARS, sp.scale, R * sizeof(double));
+    set_view(ctx, S_COEF, S_SCALARS, sp.coef, R * sizeof(double));
+    set_view(ctx, S_OUTER, S_SCALARS, sp.outer, R * sizeof(int));
     if ((s = ensure(ctx, ctx->pool[S_QSUM], R * sizeof(double2))) != DDA_OK) return s;
     if ((s = ensure(ctx, ctx->pool[S_COUNT], sizeof(int))) != DDA_OK) return s;
     return DDA_OK;
@@ -897,8 +1033,24 @@ dda_status solve_core(dda_ctx* ctx, int R, const dda_opts& o, bool refine, bool 
     double2* part = slot<double2>(ctx, S_PART);
     unsigned* cnt = slot<unsigned>(ctx, S_CNT);
     int* outer = slot<int>(ctx, S_OUTER);
-    std::vector<double> hb(R), hr(R), tmp(R);
     std::vector<int> hact(R, 1);
+    // the scalars' host copy: the staging area, or (very many RHS) a buffer of this solve
+    const ScalarParts sp(R);
+    char* h = nullptr;
+    if ((rs = stage(ctx, sp.p.total, &h)) != DDA_OK) return rs;
+    std::vector<char> own;
+    if (h == nullptr) {
+        own.resize(sp.p.total);
+        h = own.data();
+    }
+    char* dev = static_cast<char*>(ctx->pool[S_SCALARS].p);
+    const double *hb = reinterpret_cast<double*>(h + sp.norm_b), *hr = reinterpret_cast<double*>(h + sp.norm_r);
+    KState* hst = reinterpret_cast<KState*>(h + sp.state);
+    double *tolrel = reinterpret_cast<double*>(h + sp.tolrel), *scale = reinterpret_cast<double*>(h + sp.scale),
+           *coef = reinterpret_cast<double*>(h + sp.coef);
+    auto fetch = [&](size_t from, size_t to) {
+        return cudaMemcpyAsync(h + from, dev + from, to - from, cudaMemcpyDeviceToHost, s);
+    };
 
     CU(launch_residual(R, n, E, nullptr, nullptr, slot<double>(ctx, S_NORM_B), nullptr, part, cnt, s));
     if (have_x0) {
@@ -910,8 +1062,7 @@ dda_status solve_core(dda_ctx* ctx, int R, const dda_opts& o, bool refine, bool 
         CU(cudaMemsetAsync(X, 0, vb64, s));
         CU(launch_residual(R, n, E, nullptr, Rr, slot<double>(ctx, S_NORM_R), nullptr, part, cnt, s));
     }
-    CU(cudaMemcpyAsync(hb.data(), ctx->pool[S_NORM_B].p, R * sizeof(double), cudaMemcpyDeviceToHost, s));
-    CU(cudaMemcpyAsync(hr.data(), ctx->pool[S_NORM_R].p, R * sizeof(double), cudaMemcpyDeviceToHost, s));
+    CU(fetch(sp.norm_b, sp.state));
     CU(sync_collect(ctx));
     for (int r = 0; r < R; ++r) {
         tr[r].bn = std::sqrt(hb[r]);
@@ -921,13 +1072,12 @@ dda_status solve_core(dda_ctx* ctx, int R, const dda_opts& o, bool refine, bool 
     const int max_outer = refine ? (o.max_outer > 0 ? o.max_outer : 8) : 1;
     const double floor_tol = (sizeof(T) == 4) ? (o.inner_tol > 0 ? o.inner_tol : 2e-6) : 1e-15;
     Inner<T> in = InnerSlots<T>::get(ctx);
-    std::vector<KState> hst(R);
     for (int it = 0; it < max_outer; ++it) {
         int nact = 0;
-        std::vector<double> tolrel(R, 0.0), scale(R, 0.0), coef(R, 0.0);
         for (int r = 0; r < R; ++r) {
             RhsTrack& t = tr[r];
             hact[r] = 0;
+            tolrel[r] = scale[r] = coef[r] = 0.0;
             if (t.done) continue;
             if (t.rn <= o.tol * t.bn) {
                 t.done = true;
@@ -947,15 +1097,13 @@ dda_status solve_core(dda_ctx* ctx, int R, const dda_opts& o, bool refine, bool 
             tolrel[r] = std::max(want, floor_tol);
         }
         if (nact == 0) break;
-        CU(cudaMemcpyAsync(outer, hact.data(), R * sizeof(int), cudaMemcpyHostToDevice, s));
-        CU(cudaMemcpyAsync(ctx->pool[S_TOLREL].p, tolrel.data(), R * sizeof(double), cudaMemcpyHostToDevice, s));
-        CU(cudaMemcpyAsync(ctx->pool[S_SCALE].p, scale.data(), R * sizeof(double), cudaMemcpyHostToDevice, s));
-        CU(cudaMemcpyAsync(ctx->pool[S_COEF].p, coef.data(), R * sizeof(double), cudaMemcpyHostToDevice, s));
+        std::memcpy(h + sp.outer, hact.data(), R * sizeof(int));
         for (int r = 0; r < R; ++r) {
             std::memset(&hst[r], 0, sizeof(KState));
             hst[r].maxit = std::max(1, o.maxit - tr[r].iters);
         }
-        CU(cudaMemcpyAsync(ctx->pool[S_STATE].p, hst.data(), R * sizeof(KState), cudaMemcpyHostToDevice, s));
+        // (the stream is idle here, and every pass of this loop ends with a synchronization)
+        CU(cudaMemcpyAsync(dev + sp.state, h + sp.state, sp.p.total - sp.state, cudaMemcpyHostToDevice, s));
         CU(KrylovOps<cx<T>>::to_inner(R, n, Rr, in.b, slot<double>(ctx, S_SCALE), outer, s));
         CU(KrylovOps<cx<T>>::init(R, n, in.b, in.x, in.r, in.rhat, in.p, in.v,
                                   o.solver == DDA_SOLVER_BICGSTAB ? in.s : nullptr, slot<KState>(ctx, S_STATE),
@@ -964,11 +1112,10 @@ dda_status solve_core(dda_ctx* ctx, int R, const dda_opts& o, bool refine, bool 
             CU(QmrOps<cx<T>>::init(R, n, in.r, in.s, in.rhat, in.u2, in.b, slot<KState>(ctx, S_STATE),
                                    slot<int>(ctx, S_ACTIVE), part, cnt, s));
         if ((rs = inner_solve<T>(ctx, R, o.maxit, o.use_graph != 0, o.solver)) != DDA_OK) return rs;
-        CU(cudaMemcpyAsync(hst.data(), ctx->pool[S_STATE].p, R * sizeof(KState), cudaMemcpyDeviceToHost, s));
         CU(KrylovOps<cx<T>>::accumulate(R, n, X, in.x, slot<double>(ctx, S_COEF), outer, s));
         if ((rs = matvec64(ctx, R, X, Y, outer, df_resid)) != DDA_OK) return rs;
         CU(launch_residual(R, n, E, Y, Rr, slot<double>(ctx, S_NORM_R), outer, part, cnt, s));
-        CU(cudaMemcpyAsync(hr.data(), ctx->pool[S_NORM_R].p, R * sizeof(double), cudaMemcpyDeviceToHost, s));
+        CU(fetch(sp.norm_r, sp.tolrel));
         CU(sync_collect(ctx));
         for (int r = 0; r < R; ++r) {
             if (!hact[r]) continue;
@@ -1299,6 +1446,8 @@ dda_status dda_destroy(dda_ctx* ctx) {
         free_mem(ctx->m_twdf[a]);
     }
     ctx->prof.release();
+    if (ctx->stage_ev) cudaEventDestroy(ctx->stage_ev);
+    if (ctx->h_stage) cudaFreeHost(ctx->h_stage);
     if (ctx->h_count) cudaFreeHost(ctx->h_count);
     if (ctx->own_stream) cudaStreamDestroy(ctx->own_stream);
     delete ctx;
@@ -1504,6 +1653,8 @@ dda_status dda_prepare(dda_ctx* ctx, double lambda_vac, double aeff, dda_precisi
     dda_status s;
     const int Ls[3] = {g.Lx, g.Ly, g.Lz};
     for (int a = 0; a < 3; ++a) {
+        if (ctx->tw_len[a] == Ls[a]) continue;  // (the tables depend on the length alone)
+        ctx->tw_len[a] = 0;
         std::vector<double2> t64;
         std::vector<float2> t32;
         host_twiddles(Ls[a], t64, t32);
@@ -1515,16 +1666,16 @@ dda_status dda_prepare(dda_ctx* ctx, double lambda_vac, double aeff, dda_precisi
         for (size_t i = 0; i < t64.size(); ++i) tdf[i] = cdfl{dfl(t64[i].x), dfl(t64[i].y)};
         if ((s = ensure(ctx, ctx->m_twdf[a], tdf.size() * sizeof(cdfl))) != DDA_OK) return s;
         CU(cudaMemcpy(ctx->m_twdf[a].p, tdf.data(), tdf.size() * sizeof(cdfl), cudaMemcpyHostToDevice));
+        ctx->tw_len[a] = Ls[a];
     }
     const int64_t oct = 6 * g.oct_per_comp();
     if ((s = ensure(ctx, ctx->m_gh64, oct * sizeof(double2))) != DDA_OK) return s;
-    DevMem scratch;
     const size_t sb = (size_t)green_scratch_size(g) * sizeof(double2);
-    cudaError_t e = cudaMalloc(&scratch.p, sb);
-    if (e != cudaSuccess) return ctx->cuda_fail(e, "cudaMalloc(Green tensor scratch)");
-    e = launch_green_fft(g, ctx->kd, (double2*)scratch.p, (double2*)ctx->m_gh64.p, tw_of<double>(ctx), ctx->stream);
+    if ((s = ensure_scratch(ctx, ctx->pool[S_GREEN], sb)) != DDA_OK) return s;
+    cudaError_t e = launch_green_fft(g, ctx->kd, slot<double2>(ctx, S_GREEN), (double2*)ctx->m_gh64.p,
+                                     tw_of<double>(ctx), ctx->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
-    cudaFree(scratch.p);
+    if (sb > kKeepMax) free_mem(ctx->pool[S_GREEN]);
     if (e != cudaSuccess) return ctx->cuda_fail(e, "Green tensor FFT");
     ctx->has32 = false;
     if (precision != DDA_FP64) {
@@ -1573,6 +1724,9 @@ dda_status dda_solve(dda_ctx* ctx, dda_precision precision, int R, const double*
     if (st != DDA_OK && st != DDA_ERR_NOT_CONVERGED && st != DDA_ERR_BREAKDOWN) return st;
     if (P_out) {
         const size_t bytes = (size_t)R * 3 * ctx->g.N * sizeof(double2);
+        PageIn pages;
+        pages.start(P_out, bytes);
+        pages.wait();
         CU(cudaMemcpyAsync(P_out, ctx->pool[S_X64].p, bytes, cudaMemcpyDeviceToHost, ctx->stream));
         CU(sync_collect(ctx));
     }
@@ -1733,15 +1887,14 @@ dda_status nf_box(dda_ctx* ctx, const double* ext, int dims[3], int off[3]) {
     return DDA_OK;
 }
 
-struct NearWork {
-    std::vector<DevMem> mem;
-    ~NearWork() {
-        for (auto& m : mem) free_mem(m);
-    }
-    void* get(size_t bytes, cudaError_t& e) {
-        mem.emplace_back();
-        e = cudaMalloc(&mem.back().p, bytes < 256 ? 256 : bytes);
-        return mem.back().p;
+// Gives the field calls' workspace back where it is too large to keep.
+struct ScratchGuard {
+    dda_ctx* ctx;
+    explicit ScratchGuard(dda_ctx* c) : ctx(c) {}
+    ~ScratchGuard() {
+        if (ctx->pool[S_FIELD].bytes <= kKeepMax) return;
+        cudaStreamSynchronize(ctx->stream);
+        free_mem(ctx->pool[S_FIELD]);
     }
 };
 
@@ -1764,82 +1917,68 @@ dda_status nearfield_run(dda_ctx* ctx, int R, const double* P_host, const int di
     const int64_t Ne = (int64_t)dims[0] * dims[1] * dims[2], M = g.M(), N = ctx->g.N;
     if (M > (int64_t)INT32_MAX) return ctx->fail(DDA_ERR_SIZE, "extended volume too large");
     g.N = Ne;
-    std::vector<int> site_of(M, -1), lat_of(Ne);
-    for (int iz = 0; iz < dims[2]; ++iz)
-        for (int iy = 0; iy < dims[1]; ++iy)
-            for (int ix = 0; ix < dims[0]; ++ix) {
-                const int64_t b = ((int64_t)iz * dims[1] + iy) * dims[0] + ix;
-                const int64_t li = ((int64_t)iz * g.ny + iy) * g.nx + ix;
-                site_of[li] = (int)b;
-                lat_of[b] = (int)li;
-            }
-    // target site -> box point (target lattice indices from the context's map)
-    std::vector<int> tlat(N), box_of(N);
-    CU(cudaMemcpy(tlat.data(), ctx->tg.lat_of, N * sizeof(int), cudaMemcpyDeviceToHost));
-    for (int64_t j = 0; j < N; ++j) {
-        const int l = tlat[j];
-        const int ix = l % ctx->g.nx, iy = (l / ctx->g.nx) % ctx->g.ny, iz = l / (ctx->g.nx * ctx->g.ny);
-        box_of[j] = (int)(((int64_t)(iz + off[2]) * dims[1] + (iy + off[1])) * dims[0] + (ix + off[0]));
-    }
-    NearWork w;
-    cudaError_t ce = cudaSuccess;
-    auto alloc = [&](size_t bytes) { return ce == cudaSuccess ? w.get(bytes, ce) : nullptr; };
-    int* d_site = (int*)alloc(M * sizeof(int));
-    int* d_lat = (int*)alloc(Ne * sizeof(int));
-    int* d_box = (int*)alloc(N * sizeof(int));
-    uint8_t* d_comp = (uint8_t*)alloc(Ne);
-    const int64_t oct = 6 * g.oct_per_comp();
-    double2* gh64 = (double2*)alloc(oct * sizeof(double2));
-    double2* tw64[3];
-    void* twT[3];
-    for (int a = 0; a < 3; ++a) {
-        const int L = a == 0 ? g.Lx : (a == 1 ? g.Ly : g.Lz);
-        tw64[a] = (double2*)alloc(L * sizeof(double2));
-        twT[a] = sizeof(T) == 8 ? (void*)tw64[a] : alloc(L * sizeof(C));
-    }
-    C* ghT = sizeof(T) == 8 ? (C*)gh64 : (C*)alloc(oct * sizeof(C));
+    PageIn pages;  // (while the device works)
+    pages.start(Esca_out, (size_t)R * 3 * Ne * sizeof(double2));
+    pages.start(Einc_out, (size_t)R * 3 * Ne * sizeof(double2));
     const int rc = std::max(1, std::min(R, 8));  // RHS per pass over the box
-    C* Pbox = (C*)alloc((size_t)rc * 3 * Ne * sizeof(C));
-    C* Ybox = (C*)alloc((size_t)rc * 3 * Ne * sizeof(C));
-    C* u2 = (C*)alloc((size_t)rc * 3 * g.u2_per_comp() * sizeof(C));
-    C* beta0 = (C*)alloc((size_t)rc * 2 * sizeof(C));
-    double2* d_P = (double2*)alloc((size_t)rc * 3 * N * sizeof(double2));
-    double2* d_E = (double2*)alloc((size_t)rc * 3 * Ne * sizeof(double2));
-    double* d_k = (double*)alloc((size_t)R * 3 * sizeof(double));
-    double2* d_e = (double2*)alloc((size_t)R * 3 * sizeof(double2));
-    if (ce != cudaSuccess) return ctx->cuda_fail(ce, "near-field workspace");
-    CU(cudaMemcpy(d_site, site_of.data(), M * sizeof(int), cudaMemcpyHostToDevice));
-    CU(cudaMemcpy(d_lat, lat_of.data(), Ne * sizeof(int), cudaMemcpyHostToDevice));
-    CU(cudaMemcpy(d_box, box_of.data(), N * sizeof(int), cudaMemcpyHostToDevice));
-    CU(cudaMemset(d_comp, 1, Ne));
-    CU(cudaMemset(beta0, 0, (size_t)rc * 2 * sizeof(C)));
-    std::vector<double2> e2(3 * (size_t)R);
-    for (size_t i = 0; i < e2.size(); ++i) e2[i] = make_double2(e[i].real(), e[i].imag());
-    CU(cudaMemcpy(d_k, khat.data(), khat.size() * sizeof(double), cudaMemcpyHostToDevice));
-    CU(cudaMemcpy(d_e, e2.data(), e2.size() * sizeof(double2), cudaMemcpyHostToDevice));
+    const int64_t oct = 6 * g.oct_per_comp();
+    const int Ls[3] = {g.Lx, g.Ly, g.Lz};
+    // one workspace; first what comes from the host, in one copy
+    Parts parts;
+    size_t o_tw64[3], o_twT[3];
     for (int a = 0; a < 3; ++a) {
-        const int L = a == 0 ? g.Lx : (a == 1 ? g.Ly : g.Lz);
+        o_tw64[a] = parts.add(Ls[a] * sizeof(double2));
+        o_twT[a] = sizeof(T) == 8 ? o_tw64[a] : parts.add(Ls[a] * sizeof(C));
+    }
+    const size_t o_k = parts.add((size_t)R * 3 * sizeof(double)), o_e = parts.add((size_t)R * 3 * sizeof(double2));
+    const size_t host_bytes = parts.total;
+    const size_t o_site = parts.add(M * sizeof(int)), o_lat = parts.add(Ne * sizeof(int)),
+                 o_box = parts.add(N * sizeof(int)), o_comp = parts.add(Ne), o_gh = parts.add(oct * sizeof(double2)),
+                 o_ghT = sizeof(T) == 8 ? o_gh : parts.add(oct * sizeof(C)),
+                 o_P = parts.add((size_t)rc * 3 * Ne * sizeof(C)), o_Y = parts.add((size_t)rc * 3 * Ne * sizeof(C)),
+                 o_u = parts.add((size_t)rc * 3 * g.u2_per_comp() * sizeof(C)),
+                 o_beta = parts.add((size_t)rc * 2 * sizeof(C)),
+                 o_Pin = parts.add((size_t)rc * 3 * N * sizeof(double2)),
+                 o_E = parts.add((size_t)rc * 3 * Ne * sizeof(double2)),
+                 o_green = parts.add((size_t)green_scratch_size(g) * sizeof(double2));
+    dda_status ws;
+    if ((ws = ensure_scratch(ctx, ctx->pool[S_FIELD], parts.total)) != DDA_OK) return ws;
+    ScratchGuard guard(ctx);
+    char* base = slot<char>(ctx, S_FIELD);
+    int *d_site = (int*)(base + o_site), *d_lat = (int*)(base + o_lat), *d_box = (int*)(base + o_box);
+    uint8_t* d_comp = (uint8_t*)(base + o_comp);
+    double2* gh64 = (double2*)(base + o_gh);
+    C *ghT = (C*)(base + o_ghT), *Pbox = (C*)(base + o_P), *Ybox = (C*)(base + o_Y), *u2 = (C*)(base + o_u),
+      *beta0 = (C*)(base + o_beta);
+    double2 *d_P = (double2*)(base + o_Pin), *d_E = (double2*)(base + o_E), *d_e = (double2*)(base + o_e);
+    double* d_k = (double*)(base + o_k);
+    const double2* tw64[3];
+    const C* twT[3];
+    std::vector<char> hv(host_bytes);
+    char* h = hv.data();
+    for (int a = 0; a < 3; ++a) {
         std::vector<double2> t64;
         std::vector<float2> t32;
-        host_twiddles(L, t64, t32);
-        CU(cudaMemcpy(tw64[a], t64.data(), L * sizeof(double2), cudaMemcpyHostToDevice));
-        if (sizeof(T) != 8) CU(cudaMemcpy(twT[a], t32.data(), L * sizeof(float2), cudaMemcpyHostToDevice));
+        host_twiddles(Ls[a], t64, t32);
+        std::memcpy(h + o_tw64[a], t64.data(), Ls[a] * sizeof(double2));
+        if (sizeof(T) != 8) std::memcpy(h + o_twT[a], t32.data(), Ls[a] * sizeof(float2));
+        tw64[a] = (const double2*)(base + o_tw64[a]);
+        twT[a] = (const C*)(base + o_twT[a]);
     }
-    {
-        DevMem scratch;
-        CU(cudaMalloc(&scratch.p, (size_t)green_scratch_size(g) * sizeof(double2)));
-        Twiddles<double> t{tw64[0], tw64[1], tw64[2]};
-        cudaError_t e1 = launch_green_fft(g, ctx->kd, (double2*)scratch.p, gh64, t, st);
-        if (e1 == cudaSuccess) e1 = cudaStreamSynchronize(st);
-        cudaFree(scratch.p);
-        if (e1 != cudaSuccess) return ctx->cuda_fail(e1, "near-field Green tensor FFT");
-    }
+    std::memcpy(h + o_k, khat.data(), khat.size() * sizeof(double));
+    for (size_t i = 0; i < 3 * (size_t)R; ++i) ((double2*)(h + o_e))[i] = make_double2(e[i].real(), e[i].imag());
+    CU(cudaMemcpyAsync(base, h, host_bytes, cudaMemcpyHostToDevice, st));
+    CU(cudaMemsetAsync(d_comp, 1, Ne, st));
+    CU(cudaMemsetAsync(beta0, 0, (size_t)rc * 2 * sizeof(C), st));
+    CU(launch_box_maps(g, dims, d_site, d_lat, st));
+    CU(launch_box_sites(ctx->g, N, ctx->tg.lat_of, dims, off, d_box, st));
+    CU(launch_green_fft(g, ctx->kd, (double2*)(base + o_green), gh64, Twiddles<double>{tw64[0], tw64[1], tw64[2]}, st));
     if (sizeof(T) != 8) CU(launch_convert_c128_to_c64(gh64, (float2*)ghT, oct, st));
     DevTarget tg;
     tg.site_of = d_site;
     tg.lat_of = d_lat;
     tg.comp_of = d_comp;
-    Twiddles<T> tw{(const C*)twT[0], (const C*)twT[1], (const C*)twT[2]};
+    Twiddles<T> tw{twT[0], twT[1], twT[2]};
     PadWork<T> pw{nullptr, u2};
     pw.slices = ctx->force_slices != 0;
     // phase origin: the target's own centre, in box index space
@@ -1855,6 +1994,7 @@ dda_status nearfield_run(dda_ctx* ctx, int R, const double* P_host, const int di
         // y = sum_{l != j} A_jl P_l: the matvec on the box with 1/alpha = 0
         CU(launch_matvec<T>(g, rn, Pbox, Ybox, pw, tg, beta0, 2, ghT, tw, nullptr, st));
         CU(launch_negate_c128<C>((int64_t)nb, Ybox, d_E, st));
+        pages.wait();
         CU(cudaMemcpyAsync(Esca_out + (size_t)r0 * 6 * Ne, d_E, nb * sizeof(double2), cudaMemcpyDeviceToHost, st));
         if (Einc_out) {
             CU(launch_einc_at(rn, Ne, d_lat, g.nx, g.ny, cx, cy, cz, ctx->kd, d_k + 3 * r0, d_e + 3 * r0, d_E, st));
@@ -1996,14 +2136,17 @@ dda_status farfield_run(dda_ctx* ctx, int R, const std::vector<double>& khat, co
     }
     FarGeom f{g.ox, g.oy, g.oz, ndir, far_padded(ndir)};
     const size_t ntab = (size_t)groups * f.Lt() * f.ndp;
-    NearWork w;
-    cudaError_t ce = cudaSuccess;
-    auto alloc = [&](size_t bytes) { return ce == cudaSuccess ? w.get(bytes, ce) : nullptr; };
-    double2* d_P = (double2*)alloc((size_t)R * 3 * N * sizeof(double2));
-    C* d_tabs = (C*)alloc(ntab * sizeof(C));
-    double* d_dirs = (double*)alloc(dirs.size() * sizeof(double));
-    double2* d_F = (double2*)alloc((size_t)R * ndir * 3 * sizeof(double2));
-    if (ce != cudaSuccess) return ctx->cuda_fail(ce, "far-field workspace");
+    Parts parts;
+    const size_t o_P = parts.add((size_t)R * 3 * N * sizeof(double2)), o_tabs = parts.add(ntab * sizeof(C)),
+                 o_dirs = parts.add(dirs.size() * sizeof(double)),
+                 o_F = parts.add((size_t)R * ndir * 3 * sizeof(double2));
+    dda_status ws;
+    if ((ws = ensure_scratch(ctx, ctx->pool[S_FIELD], parts.total)) != DDA_OK) return ws;
+    ScratchGuard guard(ctx);
+    char* base = slot<char>(ctx, S_FIELD);
+    double2 *d_P = (double2*)(base + o_P), *d_F = (double2*)(base + o_F);
+    C* d_tabs = (C*)(base + o_tabs);
+    double* d_dirs = (double*)(base + o_dirs);
     cudaStream_t st = ctx->stream;
     CU(cudaMemcpyAsync(d_dirs, dirs.data(), dirs.size() * sizeof(double), cudaMemcpyHostToDevice, st));
     CU(launch_phase_tables<C>(f, groups, kd, d_dirs, d_tabs, st));

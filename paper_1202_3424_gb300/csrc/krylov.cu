@@ -373,6 +373,24 @@ __global__ void __launch_bounds__(kThreads)
             Pbox[((int64_t)r * 3 + c) * Ne + b] = ccast<C>(P[((int64_t)r * 3 + c) * N + j]);
     }
 }
+__global__ void __launch_bounds__(kThreads)
+    k_box_maps(int64_t M, int gx, int gy, int bx, int by, int bz, int* __restrict__ site_of, int* __restrict__ lat_of) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < M; i += (int64_t)gridDim.x * blockDim.x) {
+        const int x = (int)(i % gx), y = (int)(i / gx % gy), z = (int)(i / ((int64_t)gx * gy));
+        const bool in = x < bx && y < by && z < bz;
+        const int b = in ? (z * by + y) * bx + x : -1;
+        site_of[i] = b;
+        if (in) lat_of[b] = (int)i;
+    }
+}
+__global__ void __launch_bounds__(kThreads)
+    k_box_sites(int64_t N, const int* __restrict__ lat_of, int tx, int ty, int bx, int by, int ox, int oy, int oz,
+                int* __restrict__ box_of) {
+    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < N; j += (int64_t)gridDim.x * blockDim.x) {
+        const int l = lat_of[j], x = l % tx, y = l / tx % ty, z = l / (tx * ty);
+        box_of[j] = ((z + oz) * by + y + oy) * bx + x + ox;
+    }
+}
 // out = -(double) y  (E_sca = -sum_l A P_l)
 template <typename C>
 __global__ void __launch_bounds__(kThreads) k_negate_c128(int64_t n, const C* __restrict__ y, double2* __restrict__ out) {
@@ -380,6 +398,20 @@ __global__ void __launch_bounds__(kThreads) k_negate_c128(int64_t n, const C* __
         const double2 v = ccast<double2>(y[i]);
         out[i] = make_double2(-v.x, -v.y);
     }
+}
+cudaError_t launch_box_maps(const Geom& g, const int dims[3], int* site_of, int* lat_of, cudaStream_t s) {
+    PROF_BEGIN(s);
+    k_box_maps<<<reduce_blocks(g.M()), kThreads, 0, s>>>(g.M(), g.nx, g.ny, dims[0], dims[1], dims[2], site_of, lat_of);
+    PROF_END(KK_OTHER, 1, s);
+    return cudaGetLastError();
+}
+cudaError_t launch_box_sites(const Geom& gt, int64_t N, const int* lat_of, const int dims[3], const int off[3],
+                             int* box_of, cudaStream_t s) {
+    PROF_BEGIN(s);
+    k_box_sites<<<reduce_blocks(N), kThreads, 0, s>>>(N, lat_of, gt.nx, gt.ny, dims[0], dims[1], off[0], off[1], off[2],
+                                                      box_of);
+    PROF_END(KK_OTHER, 1, s);
+    return cudaGetLastError();
 }
 template <typename C>
 cudaError_t launch_scatter_sites(int R, int64_t N, int64_t Ne, const int* box_of, const double2* P, C* Pbox,

@@ -99,6 +99,12 @@ cudaError_t launch_einc(int R, int64_t N, const int* lat_of, const Geom& g, doub
 cudaError_t launch_einc_at(int R, int64_t N, const int* lat_of, int nx, int ny, double cx, double cy, double cz,
                            double kd, const double* khat, const double2* e, double2* E, cudaStream_t s);
 // Near field: target sites into the extended-box vector; E_sca = -y in complex128.
+// Index maps of the near-field box (dims points, every one an output site, on
+// g's extended lattice): site_of [M] and lat_of [Ne] as in DevTarget; box_of
+// [N], the box point of each site of the target gt, its (0, 0, 0) at off.
+cudaError_t launch_box_maps(const Geom& g, const int dims[3], int* site_of, int* lat_of, cudaStream_t st);
+cudaError_t launch_box_sites(const Geom& gt, int64_t N, const int* lat_of, const int dims[3], const int off[3],
+                             int* box_of, cudaStream_t st);
 template <typename C>
 cudaError_t launch_scatter_sites(int R, int64_t N, int64_t Ne, const int* box_of, const double2* P, C* Pbox,
                                  cudaStream_t s);
