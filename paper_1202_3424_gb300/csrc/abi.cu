@@ -445,7 +445,7 @@ dda_status upload_tables(dda_ctx* ctx, int R, const std::vector<double>& k, cons
     for (size_t i = 0; i < nb; ++i) {
         reinterpret_cast<double2*>(h + o64)[i] = make_double2(b[i].real(), b[i].imag());
         reinterpret_cast<float2*>(h + o32)[i] = make_float2((float)b[i].real(), (float)b[i].imag());
-        reinterpret_cast<cdfl*>(h + odf)[i] = cdfl{dfl(b[i].real()), dfl(b[i].imag())};
+        reinterpret_cast<cdfl*>(h + odf)[i] = make_cdfl(dfl(b[i].real()), dfl(b[i].imag()));
     }
     std::memcpy(h + ow, w.data(), w.size() * sizeof(double));
     std::memcpy(h + ok, k.data(), k.size() * sizeof(double));
@@ -1663,7 +1663,7 @@ dda_status dda_prepare(dda_ctx* ctx, double lambda_vac, double aeff, dda_precisi
         CU(cudaMemcpy(ctx->m_tw64[a].p, t64.data(), t64.size() * sizeof(double2), cudaMemcpyHostToDevice));
         CU(cudaMemcpy(ctx->m_tw32[a].p, t32.data(), t32.size() * sizeof(float2), cudaMemcpyHostToDevice));
         std::vector<cdfl> tdf(t64.size());
-        for (size_t i = 0; i < t64.size(); ++i) tdf[i] = cdfl{dfl(t64[i].x), dfl(t64[i].y)};
+        for (size_t i = 0; i < t64.size(); ++i) tdf[i] = make_cdfl(dfl(t64[i].x), dfl(t64[i].y));
         if ((s = ensure(ctx, ctx->m_twdf[a], tdf.size() * sizeof(cdfl))) != DDA_OK) return s;
         CU(cudaMemcpy(ctx->m_twdf[a].p, tdf.data(), tdf.size() * sizeof(cdfl), cudaMemcpyHostToDevice));
         ctx->tw_len[a] = Ls[a];

@@ -198,7 +198,7 @@ template <int SGN, typename C> struct Dft<16, SGN, C> {
         using T = typename real_of<C>::type;
         const T c1 = T(0.92387953251128675613), s1 = T(0.38268343236508977173);  // cos, sin(pi/8)
         const T r2 = T(0.70710678118654752440);
-        auto w = [](T re, T im) { C r; r.x = re; r.y = im; return r; };
+        auto w = [](T re, T im) { return cmake<C>(re, im); };
         if constexpr (J == 1) return cmul(a, w(c1, SGN > 0 ? s1 : -s1));
         else if constexpr (J == 2) return cscale(cadd(a, cmul_i<SGN>(a)), r2);
         else if constexpr (J == 3) return cmul(a, w(s1, SGN > 0 ? c1 : -c1));
@@ -259,13 +259,10 @@ template <int SGN, typename C> struct Dft<32, SGN, C> {
         using T = typename real_of<C>::type;
         if constexpr (J == 0) return a;
         else if constexpr (J == 8) return cmul_i<SGN>(a);
-        else if constexpr (J == 16) return cscale(a, T(-1));
+        else if constexpr (J == 16) return cneg(a);
         else {
             constexpr double cj = W32Table::c[J], sj = SGN > 0 ? W32Table::s[J] : -W32Table::s[J];
-            C w;
-            w.x = T(cj);
-            w.y = T(sj);
-            return cmul(a, w);
+            return cmul(a, cmake<C>(T(cj), T(sj)));
         }
     }
     template <int N2> __device__ __forceinline__ static void twiddle_row(C (&y)[8][4]) {
@@ -401,7 +398,7 @@ __device__ __forceinline__ void fft_stages(C (&v)[PL::E], int u, const C* __rest
 #pragma unroll
             for (int j = 1; j < R; ++j) {
                 w[j] = tw[j * k * STEP];
-                if constexpr (DIR > 0) w[j].y = -w[j].y;
+                if constexpr (DIR > 0) w[j] = cconj(w[j]);
             }
 #pragma unroll
             for (int q = 0; q < NB; ++q)
@@ -416,7 +413,7 @@ __device__ __forceinline__ void fft_stages(C (&v)[PL::E], int u, const C* __rest
 #pragma unroll
                 for (int j = 1; j < R; ++j) {
                     C w = tw[j * k * STEP];
-                    if constexpr (DIR > 0) w.y = -w.y;
+                    if constexpr (DIR > 0) w = cconj(w);
                     v[q * R + j] = cmul(v[q * R + j], w);
                 }
             }
@@ -489,7 +486,7 @@ __device__ __forceinline__ void fft_stages_np(C (&v)[NP][PL::E], int u, const C*
 #pragma unroll
             for (int j = 1; j < R; ++j) {
                 w[j] = tw[j * k * STEP];
-                if constexpr (DIR > 0) w[j].y = -w[j].y;
+                if constexpr (DIR > 0) w[j] = cconj(w[j]);
             }
 #pragma unroll
             for (int p = 0; p < NP; ++p)
@@ -506,7 +503,7 @@ __device__ __forceinline__ void fft_stages_np(C (&v)[NP][PL::E], int u, const C*
 #pragma unroll
                 for (int j = 1; j < R; ++j) {
                     C w = tw[j * k * STEP];
-                    if constexpr (DIR > 0) w.y = -w.y;
+                    if constexpr (DIR > 0) w = cconj(w);
 #pragma unroll
                     for (int p = 0; p < NP; ++p) v[p][q * R + j] = cmul(v[p][q * R + j], w);
                 }

@@ -396,7 +396,7 @@ __global__ void __launch_bounds__(3 * tp_z<LZ, T>() * ZPlan<LZ>::NT, zconv_min_b
                 g = gh[cc * cs + ((int64_t)kz * hy + kyo) * hx + kxo];
                 // xy is odd in x and y, xz odd in x, yz odd in y (z handled at use)
                 const bool flip = (cc == 1 && fx != fy) || (cc == 2 && fx) || (cc == 4 && fy);
-                if (flip) g = cscale(g, T(-1));
+                if (flip) g = cneg(g);
             }
             gs[(cc * HZ + kz) * SP + tt] = g;
         }
@@ -440,9 +440,9 @@ __global__ void __launch_bounds__(3 * tp_z<LZ, T>() * ZPlan<LZ>::NT, zconv_min_b
             const int kzo = fz ? LZ - kz : kz;
             C a0 = g0[kzo * SP], a1 = g1[kzo * SP], a2 = g2[kzo * SP];
             if (fz) {
-                if (z0) a0 = cscale(a0, T(-1));
-                if (z1) a1 = cscale(a1, T(-1));
-                if (z2) a2 = cscale(a2, T(-1));
+                if (z0) a0 = cneg(a0);
+                if (z1) a1 = cneg(a1);
+                if (z2) a2 = cneg(a2);
             }
             const int kr = row(kz);
             const C pa = pb[kr * SP], pbv = pb[(ROWS + kr) * SP], pc = pb[(2 * ROWS + kr) * SP];
@@ -565,7 +565,7 @@ __global__ void __launch_bounds__(zreg_threads<ZrPlan<LZ, V>>(), zreg_min_blocks
                     g = gh[cc * cs + ((int64_t)kz * hy + kyo) * hx + kxo];
                     // xy is odd in x and y, xz odd in x, yz odd in y (z handled at use)
                     const bool flip = (cc == 1 && fx != fy) || (cc == 2 && fx) || (cc == 4 && fy);
-                    if (flip) g = cscale(g, T(-1));
+                    if (flip) g = cneg(g);
                 }
                 gs[(cc * HZ + kz) * TP + tt] = g;
             }
@@ -591,7 +591,7 @@ __global__ void __launch_bounds__(zreg_threads<ZrPlan<LZ, V>>(), zreg_min_blocks
                     const bool fx = blockIdx.x * TP + tt > Lx / 2;
                     // xy is odd in x and y, xz odd in x, yz odd in y (z handled at use)
                     const bool flip = (cc == 1 && fx != fy) || (cc == 2 && fx) || (cc == 4 && fy);
-                    gs[e] = flip ? cscale(gv[q], T(-1)) : gv[q];
+                    gs[e] = flip ? cneg(gv[q]) : gv[q];
                 }
             }
         }
@@ -624,8 +624,8 @@ __global__ void __launch_bounds__(zreg_threads<ZrPlan<LZ, V>>(), zreg_min_blocks
             const C gxx = g[0], gyy = g[3 * HZ * TP], gzz = g[5 * HZ * TP];
             C gxy = g[HZ * TP], gxz = g[2 * HZ * TP], gyz = g[4 * HZ * TP];
             if (fz) {  // xz and yz are odd in z
-                gxz = cscale(gxz, T(-1));
-                gyz = cscale(gyz, T(-1));
+                gxz = cneg(gxz);
+                gyz = cneg(gyz);
             }
             const C px = vc[0][idx], py = vc[1][idx], pz = vc[2][idx];
             vc[0][idx] = cdot3(gxx, px, gxy, py, gxz, pz);
@@ -764,9 +764,9 @@ __global__ void __launch_bounds__(zreg_threads<ZrPlan<LZ, V>>(), zreg_min_blocks
             const C* g = gs + (fx ? TP - t : t) + kzo * TG;
             const C gxx = g[0], gyy = g[3 * HZ * TG], gzz = g[5 * HZ * TG];
             C gxy = g[HZ * TG], gxz = g[2 * HZ * TG], gyz = g[4 * HZ * TG];
-            if (fx != fy) gxy = cscale(gxy, T(-1));
-            if (fx != fz) gxz = cscale(gxz, T(-1));
-            if (fy != fz) gyz = cscale(gyz, T(-1));
+            if (fx != fy) gxy = cneg(gxy);
+            if (fx != fz) gxz = cneg(gxz);
+            if (fy != fz) gyz = cneg(gyz);
             const C px = vc[0][idx], py = vc[1][idx], pz = vc[2][idx];
             vc[0][idx] = cdot3(gxx, px, gxy, py, gxz, pz);
             vc[1][idx] = cdot3(gxy, px, gyy, py, gyz, pz);
