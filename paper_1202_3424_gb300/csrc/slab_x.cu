@@ -8,42 +8,48 @@ namespace dda {
 
 namespace {
 
-// Radix plan variant of the warp-local rows (XwPlan): forward, the one with the
-// fewest exchanges through shared memory; inverse, the one with the fewest
-// registers, but for 192 points, where the plan with three exchanges holds the
-// pass at its shared-memory rate (96x64x32 ellipsoid, 32 RHS: 190 us, against
-// 168 us with two).
-template <int LX> constexpr int kPlanFwd = (LX == 128 || LX == 192 || LX == 256) ? 1 : 0;
+// Radix plan variants of the warp-local rows (XwPlan), by the fused mode of the
+// matvec.  Forward: a plain gather takes the plan with the fewest exchanges
+// through shared memory; the BiCGstab gathers, which hold up to seven operands
+// per point, the one with the fewest points per lane (64 RHS of the 96x64x32
+// ellipsoid 329 us, against 393; 64^3 sphere, 2 RHS 20.5 against 23.7 us).
+// Inverse: the fewest points per lane, but for 192 points, where the plan with
+// three exchanges stays at its shared-memory rate (the ellipsoid in a solve
+// 412 us, against 354 with two exchanges; plain, 32 RHS, 190 against 168).
+template <int LX, int MODE> constexpr int kPlanFwd = MODE == 0 && (LX == 128 || LX == 192 || LX == 256) ? 1 : 0;
 template <int LX> constexpr int kPlanInv = LX == 192 ? 1 : 0;
 
-template <int LX>
-cudaError_t xfwd(const Geom& g, int R, float2* x, float2* u, const DevTarget& tg, const float2* tw, const int* active,
-                 const FusedKrylov<float>& fk, cudaStream_t st) {
-    constexpr int V = kPlanFwd<LX>;
+template <int LX, int MODE>
+cudaError_t xfwd_mode(const Geom& g, int R, float2* x, float2* u, const DevTarget& tg, const float2* tw,
+                      const int* active, const FusedKrylov<float>& fk, cudaStream_t st) {
+    constexpr int V = kPlanFwd<LX, MODE>;
     using PL = XwPlan<LX, V>;
     const size_t sm = xw_tile_bytes<PL>(xw_rows<PL>()) + (xw_shared_twiddles<LX>() ? LX * sizeof(float2) : 0);
     const int nrows = g.ny * g.nz;
     dim3 grid((nrows + xw_rows<PL>() - 1) / xw_rows<PL>(), 3, R);
     RowMap rm = row_map(g);
     rm.pitch = nrows;
-    auto go = [&](auto kern) -> cudaError_t {
-        cudaError_t e = allow_smem(kern, sm);
-        if (e != cudaSuccess) return e;
-        PROF_BEGIN(st);
-        kern<<<grid, kXwThreads, sm, st>>>(x, u, rm, tg.site_of, nrows, g.N, tw, active, fwd_vecs(fk));
-        PROF_END(KK_XFWD_C64, R, st);
-        return cudaGetLastError();
-    };
-    if (fk.mode == 0) return go(k_xfwd_w<LX, V, 0, true>);
-    if (fk.mode == 1) return go(k_xfwd_w<LX, V, 1, true>);
-    if (fk.mode == 2) return go(k_xfwd_w<LX, V, 2, true>);
-    return go(k_xfwd_w<LX, V, 3, true>);
+    cudaError_t e = allow_smem(k_xfwd_w<LX, V, MODE, true>, sm);
+    if (e != cudaSuccess) return e;
+    PROF_BEGIN(st);
+    k_xfwd_w<LX, V, MODE, true><<<grid, kXwThreads, sm, st>>>(x, u, rm, tg.site_of, nrows, g.N, tw, active,
+                                                              fwd_vecs(fk));
+    PROF_END(KK_XFWD_C64, R, st);
+    return cudaGetLastError();
+}
+template <int LX>
+cudaError_t xfwd(const Geom& g, int R, float2* x, float2* u, const DevTarget& tg, const float2* tw, const int* active,
+                 const FusedKrylov<float>& fk, cudaStream_t st) {
+    if (fk.mode == 0) return xfwd_mode<LX, 0>(g, R, x, u, tg, tw, active, fk, st);
+    if (fk.mode == 1) return xfwd_mode<LX, 1>(g, R, x, u, tg, tw, active, fk, st);
+    if (fk.mode == 2) return xfwd_mode<LX, 2>(g, R, x, u, tg, tw, active, fk, st);
+    return xfwd_mode<LX, 3>(g, R, x, u, tg, tw, active, fk, st);
 }
 
-template <int LX>
-cudaError_t xinv(const Geom& g, int R, const float2* u, float2* y, const float2* x, const DevTarget& tg,
-                 const float2* beta, int beta_stride, bool tensor, const float2* tw, int* active,
-                 const FusedKrylov<float>& fk, cudaStream_t st) {
+template <int LX, int MODE, int DIAG>
+cudaError_t xinv_mode(const Geom& g, int R, const float2* u, float2* y, const float2* x, const DevTarget& tg,
+                      const float2* beta, int beta_stride, const float2* tw, int* active,
+                      const FusedKrylov<float>& fk, cudaStream_t st) {
     constexpr int V = kPlanInv<LX>;
     using PL = XwPlan<LX, V>;
     const size_t sm = xw_tile_bytes<PL>(xwi_rows<PL>());
@@ -51,28 +57,30 @@ cudaError_t xinv(const Geom& g, int R, const float2* u, float2* y, const float2*
     dim3 grid((nrows + xwi_rows<PL>() - 1) / xwi_rows<PL>(), 3, R);
     RowMap rm = row_map(g);
     rm.pitch = g.ny * g.nz;
-    auto go = [&](auto kern) -> cudaError_t {
-        cudaError_t e = allow_smem(kern, sm);
-        if (e != cudaSuccess) return e;
-        PROF_BEGIN(st);
-        kern<<<grid, kXwiThreads, sm, st>>>(u, rm, y, x, tg.site_of, tg.comp_of, beta, beta_stride, tg.rows, nrows,
-                                            g.N, tw, active, fk.rhat, fk.st, fk.part, fk.cnt, fk.part_stride);
-        PROF_END(KK_XINV_C64, R, st);
-        return cudaGetLastError();
-    };
+    cudaError_t e = allow_smem(k_xinv_w<LX, V, MODE, DIAG, true>, sm);
+    if (e != cudaSuccess) return e;
+    PROF_BEGIN(st);
+    k_xinv_w<LX, V, MODE, DIAG, true><<<grid, kXwiThreads, sm, st>>>(u, rm, y, x, tg.site_of, tg.comp_of, beta,
+                                                                     beta_stride, tg.rows, nrows, g.N, tw, active,
+                                                                     fk.rhat, fk.st, fk.part, fk.cnt, fk.part_stride);
+    PROF_END(KK_XINV_C64, R, st);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    return fused_finalize<float>(fk.mode, R, (int)(grid.x * grid.y), fk, active, st);
+}
+template <int LX>
+cudaError_t xinv(const Geom& g, int R, const float2* u, float2* y, const float2* x, const DevTarget& tg,
+                 const float2* beta, int beta_stride, const float2* tw, int* active, const FusedKrylov<float>& fk,
+                 cudaStream_t st) {
     auto by_mode = [&](auto d) -> cudaError_t {
         constexpr int D = decltype(d)::value;
         const int mode = inverse_mode(fk.mode);
-        if (mode == 0) return go(k_xinv_w<LX, V, 0, D, true>);
-        if (mode == 1) return go(k_xinv_w<LX, V, 1, D, true>);
-        return go(k_xinv_w<LX, V, 2, D, true>);
+        if (mode == 0) return xinv_mode<LX, 0, D>(g, R, u, y, x, tg, beta, beta_stride, tw, active, fk, st);
+        if (mode == 1) return xinv_mode<LX, 1, D>(g, R, u, y, x, tg, beta, beta_stride, tw, active, fk, st);
+        return xinv_mode<LX, 2, D>(g, R, u, y, x, tg, beta, beta_stride, tw, active, fk, st);
     };
-    cudaError_t e;
-    if (tensor) e = by_mode(std::integral_constant<int, kDiagTensor>{});
-    else if (tg.comp_of == nullptr) e = by_mode(std::integral_constant<int, kDiagSite>{});
-    else e = by_mode(std::integral_constant<int, kDiagComp>{});
-    if (e != cudaSuccess) return e;
-    return fused_finalize<float>(fk.mode, R, (int)(grid.x * grid.y), fk, active, st);
+    // (anisotropic materials keep the separate passes)
+    if (tg.comp_of == nullptr) return by_mode(std::integral_constant<int, kDiagSite>{});
+    return by_mode(std::integral_constant<int, kDiagComp>{});
 }
 
 using SlabFn = cudaError_t (*)(const Geom&, int, float2*, const float4*, const Twiddles<float>&, const int*,
@@ -115,10 +123,10 @@ cudaError_t launch_slab_matvec(const Geom& g, int R, float2* x, float2* y, const
                                const float2* beta, int beta_stride, const Twiddles<float>& tw, int* active,
                                const FusedKrylov<float>& fk, cudaStream_t st) {
     SlabFn slab = slab_fn(g);
-    if (slab == nullptr) return cudaErrorInvalidValue;
+    if (slab == nullptr || w.beta_tensor) return cudaErrorInvalidValue;
     auto fwdx = [&]() -> cudaError_t { DDA_DISPATCH_L(g.Lx, xfwd, g, R, x, w.u2, tg, tw.x, active, fk, st); };
     auto invx = [&]() -> cudaError_t {
-        DDA_DISPATCH_L(g.Lx, xinv, g, R, w.u2, y, x, tg, beta, beta_stride, w.beta_tensor, tw.x, active, fk, st);
+        DDA_DISPATCH_L(g.Lx, xinv, g, R, w.u2, y, x, tg, beta, beta_stride, tw.x, active, fk, st);
     };
     cudaError_t e;
     if ((e = fwdx()) != cudaSuccess) return e;
