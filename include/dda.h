@@ -337,9 +337,9 @@ dda_status dda_grad_qabs(dda_ctx* ctx, dda_precision precision, const double* kh
  *    8 x 8 x 3, 16 x 16).
  * Where no setter below asks for anything, complex64 matvecs whose Ly and Lz
  * are at most 128 run the slab pass instead: the y and z transforms and the
- * product in one kernel over the kx planes, between x passes of its own, for
- * every RHS count and without timing anything (anisotropic materials keep the
- * passes above).  The queries below still report, and make, the choices the
+ * product in one kernel over the kx planes, between x passes of its own, without
+ * timing anything (anisotropic materials, and a few shapes for which they are
+ * faster, keep the passes above).  The queries below still report, and make, the choices the
  * separate passes would run with; launch tracing counts a slab pass as a z
  * pass with empty y passes, and once more as "slab_c64".
  * All choices compute the same product; results agree to rounding.  In

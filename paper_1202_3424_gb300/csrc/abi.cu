@@ -690,23 +690,35 @@ dda_status pick_schedule(dda_ctx* ctx, int R, bool may_time, PadWork<T>* out, bo
     return DDA_OK;
 }
 
-// The passes of a matvec of R right-hand sides: the slab pass (slab.cuh) where
-// it is built and no setter asks for a schedule of the separate passes (which
-// it replaces), else pick_schedule's choice.  Whole matvecs, separate passes ->
-// slab (sum of the kernels): 96x64x32 ellipsoid, 32 RHS 931 -> 763 us; 64^3
-// sphere, 2 RHS 109 -> 90 us; 48^3, 4 RHS 134 -> 108 us; 32^3, 8 RHS 66 -> 53 us.
-// Anisotropic materials keep the separate passes: solves of strongly absorbing
-// crystals amplify a change of rounding until single elements of P differ by
-// 1e-3 at tolerance 1e-5 (BiCGstab(2), 65 cycles), and their users compare runs.
-bool uses_slab(const dda_ctx* ctx) {
-    return slab_built(ctx->g) && !ctx->aniso && ctx->force_z < 0 && ctx->force_xf < 0 && ctx->force_xi < 0 &&
-           ctx->force_y < 0 && ctx->force_slices == 0;
+// Whether complex64 matvecs of R right-hand sides run the slab pass (slab.cuh):
+// where it is built and no setter asks for a schedule of the separate passes,
+// which it replaces.  Whole products, separate passes / slab: 96x64x32 ellipsoid,
+// 32 RHS 931 / 763 us; 64^3 sphere, 2 RHS 109 / 90 us; 48^3, 4 RHS 134 / 108 us; over
+// padded lengths 32..128 (x to 256) and 1, 3 and 12 RHS 1.0-1.45 times faster, but
+// for these, which keep the separate passes:
+//   many long, thin slabs, whose x passes, faster row by row, are most of the
+//   work: 256x48x32 padded, 12 RHS 119 / 125 us; 128x32x48 97 / 103 us;
+//   a few large slabs, which occupy a fifth of the SMs: 32x128x96 padded, 1 RHS
+//   54 / 58 us;
+//   anisotropic materials: solves of strongly absorbing crystals amplify a change
+//   of rounding until single elements of P differ by 1e-3 at tolerance 1e-5
+//   (BiCGstab(2), 65 cycles), and their users compare runs.
+bool uses_slab(const dda_ctx* ctx, int R) {
+    if (ctx->aniso || ctx->force_z >= 0 || ctx->force_xf >= 0 || ctx->force_xi >= 0 || ctx->force_y >= 0 ||
+        ctx->force_slices != 0 || !slab_built(ctx->g))
+        return false;
+    const Geom& g = ctx->g;
+    const int64_t slabs = (int64_t)g.Lx * R, points = (int64_t)g.Ly * g.Lz;
+    if (slabs >= 1024 && g.Lx >= 128 && points <= 12 * g.Lx) return false;
+    if (slabs < 48 && points >= 64 * 96) return false;
+    return true;
 }
+// The passes of a matvec: the slab pass, or pick_schedule's choice.
 template <typename T>
 dda_status choose_passes(dda_ctx* ctx, int R, bool may_time, PadWork<T>* out, bool fused = false) {
     out->slab = nullptr;
     if constexpr (std::is_same<T, float>::value) {
-        if (uses_slab(ctx)) {
+        if (uses_slab(ctx, R)) {
             out->slab = static_cast<const float4*>(ctx->m_ghslab.p);
             return DDA_OK;
         }
@@ -1080,7 +1092,7 @@ dda_status solve_core(dda_ctx* ctx, int R, const dda_opts& o, bool refine, bool 
     // results came out up to 1.7 times further from the exact solution than the
     // separate passes' (64^3 sphere; the mean was the same).  A third costs about
     // one iteration in thirty and keeps them from it.
-    const double share = (sizeof(T) == 4 && uses_slab(ctx)) ? 1.0 / 3.0 : 0.5;
+    const double share = (sizeof(T) == 4 && uses_slab(ctx, matvec_chunk<T>(ctx, R))) ? 1.0 / 3.0 : 0.5;
     Inner<T> in = InnerSlots<T>::get(ctx);
     for (int it = 0; it < max_outer; ++it) {
         int nact = 0;

@@ -17,8 +17,8 @@
 //   B  columns (ky): all three components, FFT along z (input half zero),
 //      product, inverse FFT, lattice half kept
 //   C  rows: inverse FFT along y, lattice half stored
-// The arithmetic is packed (pair.cuh): A and C run rows iz and iz+1 in the two
-// halves, B the columns ky and Ly-ky.  These two share their Green tensor:
+// The arithmetic is packed (pair.cuh): A and C run rows iz and iz + nz/2 in the
+// two halves, B the columns ky and Ly-ky.  These two share their Green tensor:
 // its entries xy and yz change sign under ky -> -ky and the others do not, so
 // with the y component of the mirrored column negated on the way in and out
 // both halves multiply by the same six numbers.  (ky = 0 and Ly/2 are their own
@@ -58,7 +58,15 @@ template <int LZ> __host__ __device__ constexpr int col_lanes() { return ColPlan
 // rows a column steps through shift by the width of the pair group, so that
 // the lanes of a half-warp fall on different banks.
 template <int LZ> __host__ __device__ constexpr int slab_wt() { return 32 / col_lanes<LZ>(); }
-template <int LY, int LZ> __host__ __device__ constexpr int slab_rs() { return LY + slab_wt<LZ>() % 16; }
+// (adjacent lanes take slab_w adjacent pairs; of eight, the half-warps take four each)
+template <int LZ> __host__ __device__ constexpr int slab_w() { return slab_wt<LZ>() < 4 ? slab_wt<LZ>() : 4; }
+template <int LZ> __host__ __device__ constexpr int col_pair(int lane) {
+    return lane % slab_w<LZ>() + (slab_wt<LZ>() > 4 ? 4 * (lane / 16) : 0);
+}
+template <int LZ> __host__ __device__ constexpr int col_lane(int lane) {  // place in the pair: u + NT par
+    return (lane / slab_w<LZ>()) % col_lanes<LZ>();
+}
+template <int LY, int LZ> __host__ __device__ constexpr int slab_rs() { return LY + slab_w<LZ>(); }
 template <int LY, int LZ> __host__ __device__ constexpr size_t slab_smem() {
     return (size_t)3 * (LZ / 2) * slab_rs<LY, LZ>() * 8 + (size_t)(LY + LZ) * 16;
 }
@@ -73,19 +81,19 @@ template <int LY, int LZ> __host__ __device__ constexpr int slab_blocks() {
 // no more slabs than SMs)
 template <int LY, int LZ, int NB> __host__ __device__ constexpr int slab_threads() { return slab_sm_threads<LZ>() / NB; }
 
-// Row pair (rows 2q, 2q+1) of pencil rp.  The two pencils of a half-warp (8
-// lanes each) must lie 8 banks apart: neighbouring pairs do where 2 RS is 8
-// mod 16; where it is 4, pairs two apart do, so 0, 2, 1, 3 of every four.
-template <int LY, int LZ> __host__ __device__ constexpr int slab_row_pair(int rp) {
-    constexpr bool apart = RowPlan<LY>::NT == 8 && (2 * slab_rs<LY, LZ>()) % 8 == 4;
-    return apart ? (rp & ~3) | ((rp & 1) << 1) | ((rp >> 1) & 1) : rp;
+// A row pencil holds rows q and q + NZ/2, real parts of its exchanges in the one
+// and imaginary parts in the other.  The 16 / NT pencils of a half-warp must lie
+// NT banks apart; rows lie slab_w apart, so they take every (NT / slab_w)-th row.
+template <int LY, int LZ> __host__ __device__ constexpr int slab_row_step() { return RowPlan<LY>::NT / slab_w<LZ>(); }
+template <int LY, int LZ> __host__ __device__ constexpr int slab_row(int rp) {
+    constexpr int H = 16 / RowPlan<LY>::NT, D = slab_row_step<LY, LZ>();
+    static_assert(D >= 1 && (LZ / 4) % (H * D) == 0, "whole groups of rows");
+    return rp / (H * D) * (H * D) + rp % H * D + rp / H % D;
 }
 
 template <int LY, int LZ> struct RowMapY {
-    // half-warp banks: pencil p of the warp holds row pair slab_row_pair(p)
     __host__ __device__ static constexpr LaneMap map() {
-        return LaneMap{1, RowPlan<LY>::NT, 32 / RowPlan<LY>::NT, 1,
-                       2 * slab_rs<LY, LZ>() * slab_row_pair<LY, LZ>(1), 0};
+        return LaneMap{1, RowPlan<LY>::NT, 32 / RowPlan<LY>::NT, 1, slab_row_step<LY, LZ>() * slab_rs<LY, LZ>(), 0};
     }
 };
 // Slots of a column pair's exchanges: the rows of S, all three components (and
@@ -93,7 +101,7 @@ template <int LY, int LZ> struct RowMapY {
 template <int LZ> __host__ __device__ constexpr int col_room() { return 3 * (LZ / 2) / (col_split<LZ>() ? 2 : 1); }
 template <int LY, int LZ> struct ColMapZ {
     __host__ __device__ static constexpr LaneMap map() {
-        return LaneMap{slab_wt<LZ>(), 1, slab_wt<LZ>(), slab_rs<LY, LZ>(), 1, col_room<LZ>()};
+        return LaneMap{slab_w<LZ>(), 1, slab_w<LZ>(), slab_rs<LY, LZ>(), 1, col_room<LZ>()};
     }
 };
 
@@ -124,8 +132,8 @@ __global__ void k_slab_green(const double2* __restrict__ gh, float4* __restrict_
         if (i < half) {
             const int lane = (int)(k % 32);
             k /= 32;
-            ky = lane % WT;
-            lp = lane / WT;
+            ky = col_pair<LZ>(lane);
+            lp = col_lane<LZ>(lane);
         } else {
             lp = (int)(k % NL);
             k /= NL;
@@ -185,7 +193,7 @@ __global__ void __launch_bounds__(slab_threads<LY, LZ, NB>(), NB)
            const float2* __restrict__ twz, const int* __restrict__ active) {
     using PY = RowPlan<LY>;
     using PZ = ColPlan<LZ>;
-    constexpr int NY = LY / 2, NZ = LZ / 2, RS = slab_rs<LY, LZ>();
+    constexpr int NY = LY / 2, NZ = LZ / 2, RS = slab_rs<LY, LZ>(), RH = NZ / 2 * RS;
     constexpr int NTH = slab_threads<LY, LZ, NB>(), NW = NTH / 32, WT = slab_wt<LZ>();
     static_assert(NTH % 32 == 0 && (LY / 2) % WT == 0, "whole warps and whole pair groups");
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -225,7 +233,7 @@ __global__ void __launch_bounds__(slab_threads<LY, LZ, NB>(), NB)
         for (int g = warp; g * RPW < NRP; g += NW) {
             const int rp = min(g * RPW + p, NRP - 1);
             const bool ok = g * RPW + p < NRP;
-            const int c = rp / (NZ / 2), iz = 2 * slab_row_pair<LY, LZ>(rp - c * (NZ / 2));
+            const int c = rp / (NZ / 2), iz = slab_row<LY, LZ>(rp - c * (NZ / 2));
             const float sg = (fx && c == 0) ? -1.f : 1.f;
             f32x2* row = reinterpret_cast<f32x2*>(S + (c * NZ + iz) * RS);
             P2 v[1][E];
@@ -234,23 +242,23 @@ __global__ void __launch_bounds__(slab_threads<LY, LZ, NB>(), NB)
 #pragma unroll
                 for (int j = 0; j < R0 / 2; ++j) {
                     const int pos = u + q * NT + j * (LY / R0);
-                    const float2 a = upk(row[pos]), b = upk(row[RS + pos]);
+                    const float2 a = upk(row[pos]), b = upk(row[RH + pos]);
                     v[0][q * R0 + j] = P2{pk(sg * a.x, sg * b.x), pk(sg * a.y, sg * b.y)};
                 }
             auto st = [&](int s, P2 x) {
                 if (ok) {
                     row[s] = x.re;
-                    row[RS + s] = x.im;
+                    row[RH + s] = x.im;
                 }
             };
-            auto ld = [&](int s) { return P2{row[s], row[RS + s]}; };
+            auto ld = [&](int s) { return P2{row[s], row[RH + s]}; };
             pair_stages<PY, -1, 0, 1, RowMapY<LY, LZ>>(v, u, tyf, ld, st, true);
             __syncwarp();
             if (ok)
                 for_each_out<PY, -1, false>(u, [&](int idx, int pos) {
                     const float2 re = upk(v[0][idx].re), im = upk(v[0][idx].im);
                     reinterpret_cast<float2*>(row)[pos] = make_float2(re.x, im.x);
-                    reinterpret_cast<float2*>(row)[RS + pos] = make_float2(re.y, im.y);
+                    reinterpret_cast<float2*>(row)[RH + pos] = make_float2(re.y, im.y);
                 });
         }
     }
@@ -260,10 +268,10 @@ __global__ void __launch_bounds__(slab_threads<LY, LZ, NB>(), NB)
         constexpr int E = PZ::E, NT = PZ::NT, R0 = stage_radix<PZ, -1>(0), NB0 = E / R0;
         constexpr bool SPLIT = col_split<LZ>();
         constexpr int JN = SPLIT ? R0 : R0 / 2;  // inputs of a first butterfly: all of the split's n, half of Lz
-        const int t = lane % WT, u = (lane / WT) % NT, par = SPLIT ? lane / (WT * NT) : 0;
+        const int t = col_pair<LZ>(lane), u = col_lane<LZ>(lane) % NT, par = col_lane<LZ>(lane) / NT;
         const int kxo = fx ? Lx - kx : kx;
         const float4* gx = G + (int64_t)kxo * (LY / 2) * LZ * 3 + lane;
-        const float4* g0 = G + slab_green_main(Lx / 2 + 1, LY, LZ) + (int64_t)kxo * LZ * 3 + lane / WT;
+        const float4* g0 = G + slab_green_main(Lx / 2 + 1, LY, LZ) + (int64_t)kxo * LZ * 3 + col_lane<LZ>(lane);
 #pragma unroll 1
         for (int g = warp; g * WT < LY / 2; g += NW) {
             const int k0 = g * WT + t, k1 = k0 == 0 ? LY / 2 : LY - k0;
@@ -352,7 +360,7 @@ __global__ void __launch_bounds__(slab_threads<LY, LZ, NB>(), NB)
         for (int g = warp; g * RPW < NRP; g += NW) {
             const int rp = min(g * RPW + p, NRP - 1);
             const bool ok = g * RPW + p < NRP;
-            const int c = rp / (NZ / 2), iz = 2 * slab_row_pair<LY, LZ>(rp - c * (NZ / 2));
+            const int c = rp / (NZ / 2), iz = slab_row<LY, LZ>(rp - c * (NZ / 2));
             const float sg = (fx && c == 0) ? -1.f : 1.f;
             f32x2* row = reinterpret_cast<f32x2*>(S + (c * NZ + iz) * RS);
             P2 v[1][E];
@@ -361,30 +369,30 @@ __global__ void __launch_bounds__(slab_threads<LY, LZ, NB>(), NB)
 #pragma unroll
                 for (int j = 0; j < R0; ++j) {
                     const int pos = u + q * NT + j * (LY / R0);
-                    const float2 a = reinterpret_cast<float2*>(row)[pos], b = reinterpret_cast<float2*>(row)[RS + pos];
+                    const float2 a = reinterpret_cast<float2*>(row)[pos], b = reinterpret_cast<float2*>(row)[RH + pos];
                     v[0][q * R0 + j] = P2{pk(a.x, b.x), pk(a.y, b.y)};
                 }
             auto st = [&](int s, P2 x) {
                 if (ok) {
                     row[s] = x.re;
-                    row[RS + s] = x.im;
+                    row[RH + s] = x.im;
                 }
             };
-            auto ld = [&](int s) { return P2{row[s], row[RS + s]}; };
+            auto ld = [&](int s) { return P2{row[s], row[RH + s]}; };
             pair_stages<PY, +1, 0, 1, RowMapY<LY, LZ>>(v, u, tyi, ld, st, false);
             __syncwarp();
             if (ok)
                 for_each_out<PY, +1, true>(u, [&](int idx, int pos) {
                     const float2 re = upk(v[0][idx].re), im = upk(v[0][idx].im);
                     reinterpret_cast<float2*>(row)[pos] = make_float2(sg * re.x, sg * im.x);
-                    reinterpret_cast<float2*>(row)[RS + pos] = make_float2(sg * re.y, sg * im.y);
+                    reinterpret_cast<float2*>(row)[RH + pos] = make_float2(sg * re.y, sg * im.y);
                 });
             // the finished rows leave by bulk copies, one per row
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();
             if (ok && u < 2) {
-                const unsigned src = (unsigned)__cvta_generic_to_shared(row + u * RS);
-                float2* out = ub + c * cstride + (iz + u) * NY;
+                const unsigned src = (unsigned)__cvta_generic_to_shared(row + u * RH);
+                float2* out = ub + c * cstride + (iz + u * (NZ / 2)) * NY;
                 asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(out), "r"(src),
                              "r"((unsigned)(NY * 8))
                              : "memory");

@@ -17,7 +17,7 @@ namespace {
 // three exchanges stays at its shared-memory rate (the ellipsoid in a solve
 // 412 us, against 354 with two exchanges; plain, 32 RHS, 190 against 168).
 template <int LX, int MODE> constexpr int kPlanFwd = MODE == 0 && (LX == 128 || LX == 192 || LX == 256) ? 1 : 0;
-template <int LX> constexpr int kPlanInv = LX == 192 ? 1 : 0;
+template <int LX> constexpr int kPlanInv = LX == 192 || LX == 256 ? 1 : 0;
 
 template <int LX, int MODE>
 cudaError_t xfwd_mode(const Geom& g, int R, float2* x, float2* u, const DevTarget& tg, const float2* tw,
@@ -52,15 +52,16 @@ cudaError_t xinv_mode(const Geom& g, int R, const float2* u, float2* y, const fl
                       const FusedKrylov<float>& fk, cudaStream_t st) {
     constexpr int V = kPlanInv<LX>;
     using PL = XwPlan<LX, V>;
-    const size_t sm = xw_tile_bytes<PL>(xwi_rows<PL>());
+    constexpr int rows = xwi_rows<PL, true>();
+    const size_t sm = xw_tile_bytes<PL>(rows);
     const int nrows = tg.rows != nullptr ? tg.nrows : g.ny * g.nz;
-    dim3 grid((nrows + xwi_rows<PL>() - 1) / xwi_rows<PL>(), 3, R);
+    dim3 grid((nrows + rows - 1) / rows, 3, R);
     RowMap rm = row_map(g);
     rm.pitch = g.ny * g.nz;
     cudaError_t e = allow_smem(k_xinv_w<LX, V, MODE, DIAG, true>, sm);
     if (e != cudaSuccess) return e;
     PROF_BEGIN(st);
-    k_xinv_w<LX, V, MODE, DIAG, true><<<grid, kXwiThreads, sm, st>>>(u, rm, y, x, tg.site_of, tg.comp_of, beta,
+    k_xinv_w<LX, V, MODE, DIAG, true><<<grid, xwi_threads<PL, true>(), sm, st>>>(u, rm, y, x, tg.site_of, tg.comp_of, beta,
                                                                      beta_stride, tg.rows, nrows, g.N, tw, active,
                                                                      fk.rhat, fk.st, fk.part, fk.cnt, fk.part_stride);
     PROF_END(KK_XINV_C64, R, st);

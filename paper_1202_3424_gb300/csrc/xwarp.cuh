@@ -132,7 +132,13 @@ template <class PL> struct WarpSwz {
 constexpr int kXwThreads = 256;
 constexpr int kXwiThreads = 128;
 template <class PL> __host__ __device__ constexpr int xw_rows() { return kXwThreads / PL::NT; }
-template <class PL> __host__ __device__ constexpr int xwi_rows() { return kXwiThreads / PL::NT; }
+// (kx-major tiles: 16 rows where a pencil has 16 lanes too, for 128-byte segments)
+template <class PL, bool TR = false> __host__ __device__ constexpr int xwi_threads() {
+    return TR && PL::NT == 16 ? 256 : kXwiThreads;
+}
+template <class PL, bool TR = false> __host__ __device__ constexpr int xwi_rows() {
+    return xwi_threads<PL, TR>() / PL::NT;
+}
 // (the shuffle variants need no exchange plane)
 template <class PL> __host__ __device__ constexpr int xw_plane() {
     return xw_shfl<PL>::value ? 0 : PL::L + warp_plane_pad(PL::NT);
@@ -153,6 +159,7 @@ template <class PL> __host__ __device__ constexpr int xwi_min_blocks() {
 // next larger budget (85 registers at 8 points per lane, 102 at 12)
 template <class PL, int MODE, bool TR> __host__ __device__ constexpr int xwi_mode_min_blocks() {
     if (TR && PL::E > 16 && PL::E <= 24) return 4;
+    if (TR && xwi_threads<PL, TR>() == 256) return xwi_mode_min_blocks<PL, MODE, false>() / 2;
     return MODE != 2 ? xwi_min_blocks<PL>() : (PL::E <= 8 ? 6 : (PL::E <= 12 ? 5 : xwi_min_blocks<PL>()));
 }
 
@@ -277,7 +284,8 @@ __global__ void __launch_bounds__(kXwThreads, xwf_min_blocks<XwPlan<LX, V>>())
 // Same result as k_xinv (Y = conv + (1/alpha) X at the occupied sites, the
 // DIAG kinds, and the fused BiCGstab reductions of MODE 1 and 2).
 template <int LX, int V, int MODE, int DIAG, bool TR = false>
-__global__ void __launch_bounds__(kXwiThreads, (xwi_mode_min_blocks<XwPlan<LX, V>, MODE, TR>()))
+__global__ void __launch_bounds__((xwi_threads<XwPlan<LX, V>, TR>()),
+                                   (xwi_mode_min_blocks<XwPlan<LX, V>, MODE, TR>()))
     k_xinv_w(const float2* __restrict__ U, RowMap rm, float2* __restrict__ Y, const float2* __restrict__ X,
              const int* __restrict__ site_of, const uint8_t* __restrict__ comp_of, const float2* __restrict__ beta,
              int beta_stride, const int* __restrict__ rows, int nrows, int64_t N, const float2* __restrict__ tw,
@@ -286,7 +294,7 @@ __global__ void __launch_bounds__(kXwiThreads, (xwi_mode_min_blocks<XwPlan<LX, V
              unsigned* __restrict__ cnt, int part_stride) {
     using C = float2;
     using PL = XwPlan<LX, V>;
-    constexpr int NT = PL::NT, E = PL::E, NX = LX / 2, RPB = xwi_rows<PL>(), PS = xw_plane<PL>();
+    constexpr int NT = PL::NT, E = PL::E, NX = LX / 2, RPB = xwi_rows<PL, TR>(), PS = xw_plane<PL>();
     constexpr int R0 = stage_radix<PL, +1>(0), NB0 = E / R0;
     constexpr int RL = stage_radix<PL, +1>(PL::NS - 1), NBL = E / RL, MN = RL / 2, NO = NBL * MN;
     extern __shared__ __align__(16) unsigned char smem_raw[];

@@ -38,7 +38,7 @@ def _clusters(nx, ny, nz, seed):
 @pytest.mark.parametrize("Lz", sorted(HALF))
 @pytest.mark.parametrize("Ly", sorted(HALF))
 def test_slab_matvec_matches_oracle(lib, Ly, Lz):
-    grid = _clusters(6, HALF[Ly], HALF[Lz], 7 * Ly + Lz)
+    grid = _clusters(20, HALF[Ly], HALF[Lz], 7 * Ly + Lz)
     ctx = lib.Context(0)
     ctx.set_target(grid)
     ctx.set_materials([2.0 + 0.5j])
@@ -50,7 +50,7 @@ def test_slab_matvec_matches_oracle(lib, Ly, Lz):
     rr, comp = oracle.site_positions(grid)
     beta = oracle.ldr_inverse_polarizability(np.full(comp.shape, (2.0 + 0.5j) ** 2), kd, k[0], e[0])
     X = random_complex((12, 3, info["ndipoles"]), 3)
-    one = ctx.matvec(2, k, e, X[:1])                       # 16 slabs: one block per SM
+    one = ctx.matvec(2, k, e, X[:1])                       # 48 slabs: one block per SM
     many = ctx.matvec(2, np.tile(k, (12, 1)), np.tile(e, (12, 1)), X)
     want = pairwise.matvec(rr, kd, beta, X[0].T)[0]
     scale = np.abs(want).max()
