@@ -86,6 +86,7 @@ struct dda_ctx {
     // per-site materials (dda_set_site_materials): m holds one index per
     // occupied site, and site j takes table entry j + 1 (tg.comp_of is null)
     bool site_mode = false;
+    DevMem m_site_index;  // the indices on the device (double2 [N])
 
     // prepared wavelength
     bool prepared = false, has32 = false;
@@ -420,40 +421,55 @@ dda_status upload_tables(dda_ctx* ctx, int R, const std::vector<double>& k, cons
     std::vector<cd> b;
     std::vector<double> w;
     dda_status s;
-    if ((s = diag_tables(ctx, R, k, e, b, &w)) != DDA_OK) return s;
-    const size_t nb = b.size();
+    const bool site = ctx->site_mode;  // those tables are formed on the device
+    if (!site && (s = diag_tables(ctx, R, k, e, b, &w)) != DDA_OK) return s;
+    const size_t nb = (size_t)R * beta_rhs_stride(ctx), nw = (size_t)R * qweight_stride(ctx);
     Parts parts;
+    const size_t ok = parts.add(k.size() * sizeof(double)), oe = parts.add(3 * (size_t)R * sizeof(double2)),
+                 oS = parts.add(R * sizeof(double)), obad = parts.add(sizeof(int));
+    size_t host_bytes = parts.total;
     const size_t o64 = parts.add(nb * sizeof(double2)), o32 = parts.add(nb * sizeof(float2)),
-                 odf = parts.add(nb * sizeof(cdfl)), ow = parts.add(w.size() * sizeof(double)),
-                 ok = parts.add(k.size() * sizeof(double)), oe = parts.add(3 * (size_t)R * sizeof(double2));
+                 odf = parts.add(nb * sizeof(cdfl)), ow = parts.add(nw * sizeof(double));
+    if (!site) host_bytes = parts.total;
     if ((s = ensure(ctx, ctx->pool[S_TABLES], parts.total)) != DDA_OK) return s;
     set_view(ctx, S_BETA64, S_TABLES, o64, nb * sizeof(double2));
     set_view(ctx, S_BETA32, S_TABLES, o32, nb * sizeof(float2));
     set_view(ctx, S_BETADF, S_TABLES, odf, nb * sizeof(cdfl));
-    set_view(ctx, S_W, S_TABLES, ow, w.size() * sizeof(double));
+    set_view(ctx, S_W, S_TABLES, ow, nw * sizeof(double));
     set_view(ctx, S_KHAT, S_TABLES, ok, k.size() * sizeof(double));
     set_view(ctx, S_EPOL, S_TABLES, oe, 3 * (size_t)R * sizeof(double2));
     // through the staging area (the caller's own synchronization ends the copy),
     // or, for tables of many sites, from a buffer of this call
     char* h = nullptr;
-    if ((s = stage(ctx, parts.total, &h)) != DDA_OK) return s;
+    if ((s = stage(ctx, host_bytes, &h)) != DDA_OK) return s;
     std::vector<char> own;
     if (h == nullptr) {
-        own.resize(parts.total);
+        own.resize(host_bytes);
         h = own.data();
     }
-    for (size_t i = 0; i < nb; ++i) {
+    for (size_t i = 0; i < b.size(); ++i) {
         reinterpret_cast<double2*>(h + o64)[i] = make_double2(b[i].real(), b[i].imag());
         reinterpret_cast<float2*>(h + o32)[i] = make_float2((float)b[i].real(), (float)b[i].imag());
         reinterpret_cast<cdfl*>(h + odf)[i] = make_cdfl(dfl(b[i].real()), dfl(b[i].imag()));
     }
-    std::memcpy(h + ow, w.data(), w.size() * sizeof(double));
+    if (!site) std::memcpy(h + ow, w.data(), nw * sizeof(double));
+    for (int r = 0; r < R; ++r) reinterpret_cast<double*>(h + oS)[r] = ldr_s(&k[3 * r], &e[3 * r]);
+    *reinterpret_cast<int*>(h + obad) = 0;
     std::memcpy(h + ok, k.data(), k.size() * sizeof(double));
     for (size_t i = 0; i < 3 * (size_t)R; ++i)
         reinterpret_cast<double2*>(h + oe)[i] = make_double2(e[i].real(), e[i].imag());
-    CU(cudaMemcpyAsync(ctx->pool[S_TABLES].p, h, parts.total, cudaMemcpyHostToDevice, ctx->stream));
+    CU(cudaMemcpyAsync(ctx->pool[S_TABLES].p, h, host_bytes, cudaMemcpyHostToDevice, ctx->stream));
     if (own.empty()) CU(cudaEventRecord(ctx->stage_ev, ctx->stream));
     else CU(sync_collect(ctx));  // the buffer goes out of scope
+    if (site) {
+        char* base = slot<char>(ctx, S_TABLES);
+        CU(launch_site_tables(R, ctx->g.N, (const double2*)ctx->m_site_index.p, ctx->m_amb, ctx->kd, {kB1, kB2, kB3},
+                              (const double*)(base + oS), (double2*)(base + o64), (float2*)(base + o32),
+                              (cdfl*)(base + odf), (double*)(base + ow), (int*)(base + obad), ctx->stream));
+        CU(cudaMemcpyAsync(ctx->h_count, base + obad, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+        CU(sync_collect(ctx));
+        if (*ctx->h_count != 0) return ctx->fail(DDA_ERR_NONFINITE, "polarizability of a site is not finite");
+    }
     return DDA_OK;
 }
 
@@ -1462,6 +1478,7 @@ dda_status dda_destroy(dda_ctx* ctx) {
     free_mem(ctx->m_gh32);
     free_mem(ctx->m_ghdf);
     free_mem(ctx->m_ghslab);
+    free_mem(ctx->m_site_index);
     for (int a = 0; a < 3; ++a) {
         free_mem(ctx->m_tw64[a]);
         free_mem(ctx->m_tw32[a]);
@@ -1689,6 +1706,11 @@ dda_status dda_prepare(dda_ctx* ctx, double lambda_vac, double aeff, dda_precisi
         if ((s = ensure(ctx, ctx->m_twdf[a], tdf.size() * sizeof(cdfl))) != DDA_OK) return s;
         CU(cudaMemcpy(ctx->m_twdf[a].p, tdf.data(), tdf.size() * sizeof(cdfl), cudaMemcpyHostToDevice));
         ctx->tw_len[a] = Ls[a];
+    }
+    if (ctx->site_mode) {
+        const size_t mb = (size_t)g.N * sizeof(double2);
+        if ((s = ensure_scratch(ctx, ctx->m_site_index, mb)) != DDA_OK) return s;
+        CU(cudaMemcpy(ctx->m_site_index.p, ctx->m.data(), mb, cudaMemcpyHostToDevice));
     }
     const int64_t oct = 6 * g.oct_per_comp();
     if ((s = ensure(ctx, ctx->m_gh64, oct * sizeof(double2))) != DDA_OK) return s;
@@ -2400,14 +2422,20 @@ dda_status dda_grad_qabs(dda_ctx* ctx, dda_precision precision, const double* kh
     std::vector<cd> ev;
     if ((rs = check_rhs(ctx, 1, khat, e, k, ev)) != DDA_OK) return rs;
     const int BS = beta_stride(ctx);
-    std::vector<double2> db(BS, make_double2(0.0, 0.0));
-    for (int c = 1; c < BS; ++c) {
-        const cd mr = ctx->m[c - 1] / ctx->m_amb;
-        const cd v = ldr_inverse_alpha_deps(mr * mr, ctx->kd, k.data(), ev.data());
-        db[c] = make_double2(v.real(), v.imag());
-    }
     if ((rs = ensure(ctx, ctx->pool[S_DBETA], BS * sizeof(double2))) != DDA_OK) return rs;
-    CU(cudaMemcpyAsync(ctx->pool[S_DBETA].p, db.data(), BS * sizeof(double2), cudaMemcpyHostToDevice, ctx->stream));
+    std::vector<double2> db;
+    if (ctx->site_mode) {
+        CU(launch_site_deps(N, (const double2*)ctx->m_site_index.p, ctx->m_amb, ctx->kd, {kB1, kB2, kB3},
+                            ldr_s(k.data(), ev.data()), slot<double2>(ctx, S_DBETA), ctx->stream));
+    } else {
+        db.assign(BS, make_double2(0.0, 0.0));
+        for (int c = 1; c < BS; ++c) {
+            const cd mr = ctx->m[c - 1] / ctx->m_amb;
+            const cd v = ldr_inverse_alpha_deps(mr * mr, ctx->kd, k.data(), ev.data());
+            db[c] = make_double2(v.real(), v.imag());
+        }
+        CU(cudaMemcpyAsync(ctx->pool[S_DBETA].p, db.data(), BS * sizeof(double2), cudaMemcpyHostToDevice, ctx->stream));
+    }
     if ((rs = ensure(ctx, ctx->pool[S_MV_X32], (size_t)2 * N * sizeof(double))) != DDA_OK) return rs;
     double* g = slot<double>(ctx, S_MV_X32);
     const double K = 4.0 * ctx->kd / (ctx->aeff_lat * ctx->aeff_lat);

@@ -399,6 +399,74 @@ __global__ void __launch_bounds__(kThreads) k_negate_c128(int64_t n, const C* __
         out[i] = make_double2(-v.x, -v.y);
     }
 }
+namespace {
+// a / b, scaled against overflow
+__device__ __forceinline__ double2 zdiv_scaled(double2 a, double2 b) {
+    const double s = 1.0 / fmax(fabs(b.x), fabs(b.y));
+    const double2 bs = make_double2(b.x * s, b.y * s), as = make_double2(a.x * s, a.y * s);
+    const double d = 1.0 / (bs.x * bs.x + bs.y * bs.y);
+    return make_double2((as.x * bs.x + as.y * bs.y) * d, (as.y * bs.x - as.x * bs.y) * d);
+}
+__device__ __forceinline__ double2 site_eps(double2 m, double m_amb) {
+    const double2 r = make_double2(m.x / m_amb, m.y / m_amb);
+    return make_double2(r.x * r.x - r.y * r.y, 2.0 * r.x * r.y);
+}
+constexpr double kFourPi = 4.0 * 3.14159265358979323846;
+
+// One thread per table entry.  (Formed on the host, the tables of a 32^3
+// sphere's 17 thousand sites took 1 ms of every solve and product.)
+__global__ void __launch_bounds__(kThreads)
+    k_site_tables(int R, int64_t N, const double2* __restrict__ m, double m_amb, double kd, LdrCoeffs b,
+                  const double* __restrict__ S, double2* __restrict__ b64, float2* __restrict__ b32,
+                  cdfl* __restrict__ bdf, double* __restrict__ w, int* __restrict__ bad) {
+    const int64_t total = (int64_t)R * (N + 1);
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
+        const int r = (int)(i / (N + 1));
+        const int64_t j = i - (int64_t)r * (N + 1);
+        double2 v = make_double2(0.0, 0.0);
+        double weight = 0.0;
+        if (j > 0) {
+            const double2 e = site_eps(m[j - 1], m_amb);
+            const double2 q = zdiv_scaled(make_double2(e.x + 2.0, e.y), make_double2(e.x - 1.0, e.y));
+            const double f = b.b2 + b.b3 * S[r], k2 = kd * kd, rad = (2.0 / 3.0) * kd * kd * kd;
+            v = make_double2(kFourPi / 3.0 * q.x + (b.b1 + f * e.x) * k2, kFourPi / 3.0 * q.y + f * e.y * k2 - rad);
+            weight = -v.y - rad;
+            if (!finite2(v)) *bad = 1;
+        }
+        b64[i] = v;
+        b32[i] = make_float2((float)v.x, (float)v.y);
+        bdf[i] = ccast<cdfl>(v);
+        w[i] = weight;
+    }
+}
+__global__ void __launch_bounds__(kThreads)
+    k_site_deps(int64_t N, const double2* __restrict__ m, double m_amb, double kd, LdrCoeffs b, double S,
+                double2* __restrict__ deps) {
+    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j <= N; j += (int64_t)gridDim.x * blockDim.x) {
+        double2 v = make_double2(0.0, 0.0);
+        if (j > 0) {
+            const double2 e = site_eps(m[j - 1], m_amb), d = make_double2(e.x - 1.0, e.y);
+            const double2 q = zdiv_scaled(zdiv_scaled(make_double2(-kFourPi, 0.0), d), d);
+            v = make_double2(q.x + (b.b2 + b.b3 * S) * kd * kd, q.y);
+        }
+        deps[j] = v;
+    }
+}
+}  // namespace
+cudaError_t launch_site_tables(int R, int64_t N, const double2* m, double m_amb, double kd, LdrCoeffs b, const double* S,
+                               double2* b64, float2* b32, cdfl* bdf, double* w, int* bad, cudaStream_t s) {
+    PROF_BEGIN(s);
+    k_site_tables<<<reduce_blocks(N * R), kThreads, 0, s>>>(R, N, m, m_amb, kd, b, S, b64, b32, bdf, w, bad);
+    PROF_END(KK_OTHER, R, s);
+    return cudaGetLastError();
+}
+cudaError_t launch_site_deps(int64_t N, const double2* m, double m_amb, double kd, LdrCoeffs b, double S, double2* deps,
+                             cudaStream_t s) {
+    PROF_BEGIN(s);
+    k_site_deps<<<reduce_blocks(N), kThreads, 0, s>>>(N, m, m_amb, kd, b, S, deps);
+    PROF_END(KK_OTHER, 1, s);
+    return cudaGetLastError();
+}
 cudaError_t launch_box_maps(const Geom& g, const int dims[3], int* site_of, int* lat_of, cudaStream_t s) {
     PROF_BEGIN(s);
     k_box_maps<<<reduce_blocks(g.M()), kThreads, 0, s>>>(g.M(), g.nx, g.ny, dims[0], dims[1], dims[2], site_of, lat_of);

@@ -99,6 +99,18 @@ cudaError_t launch_einc(int R, int64_t N, const int* lat_of, const Geom& g, doub
 cudaError_t launch_einc_at(int R, int64_t N, const int* lat_of, int nx, int ny, double cx, double cy, double cz,
                            double kd, const double* khat, const double2* e, double2* E, cudaStream_t s);
 // Near field: target sites into the extended-box vector; E_sca = -y in complex128.
+// Per-site materials (N sites, refractive indices m, ambient index m_amb): the
+// LATTDR tables of upload_tables for R RHS with factors S[r] -- entry s + 1 of RHS
+// r for site s, entry 0 zero -- in FP64, FP32 and double-float, and the absorption
+// weights -Im(1/alpha) - (2/3)k^3; *bad (zeroed by the caller) is set if a value
+// is not finite.  deps: d(1/alpha)/d(eps) for one RHS, same entries.
+struct LdrCoeffs {
+    double b1, b2, b3;
+};
+cudaError_t launch_site_tables(int R, int64_t N, const double2* m, double m_amb, double kd, LdrCoeffs b, const double* S,
+                               double2* b64, float2* b32, cdfl* bdf, double* w, int* bad, cudaStream_t st);
+cudaError_t launch_site_deps(int64_t N, const double2* m, double m_amb, double kd, LdrCoeffs b, double S, double2* deps,
+                             cudaStream_t st);
 // Index maps of the near-field box (dims points, every one an output site, on
 // g's extended lattice): site_of [M] and lat_of [Ne] as in DevTarget; box_of
 // [N], the box point of each site of the target gt, its (0, 0, 0) at off.
