@@ -606,20 +606,15 @@ def read_profile(dda, ctx):
                     ("units", ctypes.c_double)]
 
     lib = dda.load_library()
-    lib.dda_profile_read.argtypes = [ctypes.c_void_p, ctypes.POINTER(Stat), ctypes.c_int, ctypes.POINTER(ctypes.c_int)]
+    lib.dda_profile_kernels.argtypes = [ctypes.c_void_p, ctypes.POINTER(Stat), ctypes.c_int, ctypes.POINTER(ctypes.c_int)]
     arr = (Stat * 64)()
     n = ctypes.c_int()
-    lib.dda_profile_read(ctx.handle, arr, 64, ctypes.byref(n))
+    lib.dda_profile_kernels(ctx.handle, arr, 64, ctypes.byref(n))
     out = {}
     total = sum(arr[i].total_ms for i in range(n.value))
     for i in range(n.value):
         out[arr[i].name.decode()] = {"launches": arr[i].launches, "ms": arr[i].total_ms, "units": arr[i].units,
                                      "share": arr[i].total_ms / total if total else 0.0}
-    # the slab pass (y and z transforms in one kernel) is traced as a z pass
-    # with empty y passes, and counted once more under its own name
-    if "slab_c64" in out and out["slab_c64"]["launches"] == out["z_conv_c64"]["launches"]:
-        out["slab_c64"] = out.pop("z_conv_c64")
-        del out["y_fwd_c64"], out["y_inv_c64"]
     return out
 
 

@@ -340,8 +340,7 @@ dda_status dda_grad_qabs(dda_ctx* ctx, dda_precision precision, const double* kh
  * product in one kernel over the kx planes, between x passes of its own, without
  * timing anything (anisotropic materials, and a few shapes for which they are
  * faster, keep the passes above).  The queries below still report, and make, the choices the
- * separate passes would run with; launch tracing counts a slab pass as a z
- * pass with empty y passes, and once more as "slab_c64".
+ * separate passes would run with.
  * All choices compute the same product; results agree to rounding.  In
  * automatic mode the context times the available choices inside whole
  * matvecs on its own workspace the first time a matvec of a given type and
@@ -388,13 +387,19 @@ dda_status dda_get_solve_schedule(dda_ctx* ctx, int R, int* zpass, int* xfwd, in
  * duration is accumulated per kernel kind.  `units` sums the right-hand sides
  * each launch processed.  Enabling resets the counters.                        */
 typedef struct {
-    char name[24];      /* kernel kind, e.g. "z_conv_c64"                                */
+    char name[24];      /* pass or kernel, e.g. "z_conv_c64"                             */
     int64_t launches;
     double total_ms;
     double units;
 } dda_kernel_stat;
 dda_status dda_profile_enable(dda_ctx* ctx, int on);
-/* Fills up to max_entries kinds that launched at least once; *n_entries = all such kinds. */
+/* Both fill up to max_entries kinds that launched at least once; *n_entries = all such kinds.
+ * dda_profile_kernels: by kernel, what was launched: a matvec through the slab
+ *   pass is three entries, "x_fwd_c64", "slab_c64" and "x_inv_c64".
+ * dda_profile_read: by pass of the matvec: a slab kernel, which carries the
+ *   y-forward, z and y-inverse passes, counts as one of each, its time under
+ *   "z_conv_c64".  Times add up to the same total either way.                   */
+dda_status dda_profile_kernels(const dda_ctx* ctx, dda_kernel_stat* out, int max_entries, int* n_entries);
 dda_status dda_profile_read(const dda_ctx* ctx, dda_kernel_stat* out, int max_entries, int* n_entries);
 
 #ifdef __cplusplus

@@ -1436,6 +1436,25 @@ void set_isotropy(dda_ctx* ctx, bool aniso) {
         ctx->graph.exec = nullptr;
     }
 }
+
+// The kinds with at least one launch, of which max_entries fit in out; how many there are.
+int profile_entries(const long long* launches, const double* ms, const double* units, dda_kernel_stat* out,
+                    int max_entries) {
+    int n = 0;
+    for (int k = 0; k < KK_COUNT; ++k) {
+        if (launches[k] == 0) continue;
+        if (n < max_entries) {
+            dda_kernel_stat& st = out[n];
+            std::memset(&st, 0, sizeof st);
+            std::snprintf(st.name, sizeof st.name, "%s", kernel_kind_name(k));
+            st.launches = launches[k];
+            st.total_ms = ms[k];
+            st.units = units[k];
+        }
+        ++n;
+    }
+    return n;
+}
 }  // namespace
 
 // ================================================================== ABI ===
@@ -2573,22 +2592,27 @@ dda_status dda_profile_enable(dda_ctx* ctx, int on) {
     return DDA_OK;
 }
 
+dda_status dda_profile_kernels(const dda_ctx* ctx, dda_kernel_stat* out, int max_entries, int* n_entries) {
+    if (!ctx || !n_entries || (max_entries > 0 && !out)) return DDA_ERR_ARG;
+    *n_entries = profile_entries(ctx->prof.launches, ctx->prof.ms, ctx->prof.unit_sum, out, max_entries);
+    return DDA_OK;
+}
+
 dda_status dda_profile_read(const dda_ctx* ctx, dda_kernel_stat* out, int max_entries, int* n_entries) {
     if (!ctx || !n_entries || (max_entries > 0 && !out)) return DDA_ERR_ARG;
-    int n = 0;
-    for (int k = 0; k < KK_COUNT; ++k) {
-        if (ctx->prof.launches[k] == 0) continue;
-        if (n < max_entries) {
-            dda_kernel_stat& st = out[n];
-            std::memset(&st, 0, sizeof st);
-            std::snprintf(st.name, sizeof st.name, "%s", kernel_kind_name(k));
-            st.launches = ctx->prof.launches[k];
-            st.total_ms = ctx->prof.ms[k];
-            st.units = ctx->prof.unit_sum[k];
-        }
-        ++n;
+    long long launches[KK_COUNT];
+    double ms[KK_COUNT], units[KK_COUNT];
+    std::copy_n(ctx->prof.launches, (int)KK_COUNT, launches);
+    std::copy_n(ctx->prof.ms, (int)KK_COUNT, ms);
+    std::copy_n(ctx->prof.unit_sum, (int)KK_COUNT, units);
+    // the passes a slab kernel carries
+    for (int pass : {KK_YFWD_C64, KK_ZCONV_C64, KK_YINV_C64}) {
+        launches[pass] += launches[KK_SLAB_C64];
+        units[pass] += units[KK_SLAB_C64];
     }
-    *n_entries = n;
+    ms[KK_ZCONV_C64] += ms[KK_SLAB_C64];
+    launches[KK_SLAB_C64] = 0;
+    *n_entries = profile_entries(launches, ms, units, out, max_entries);
     return DDA_OK;
 }
 

@@ -422,17 +422,9 @@ cudaError_t launch_slab(const Geom& g, int R, float2* u, const float4* gs, const
     const int threads = wide ? slab_threads<LY, LZ, 1>() : slab_threads<LY, LZ, NB>();
     cudaError_t e = allow_smem(kern, sm);
     if (e != cudaSuccess) return e;
-    // traced as the z pass; the y passes it carries and the slab kind itself get
-    // an entry per launch too, empty, so that every pass of a matvec counts
-    for (int kind : {KK_SLAB_C64, KK_YFWD_C64}) {
-        PROF_BEGIN(st);
-        PROF_END(kind, R, st);
-    }
     PROF_BEGIN(st);
     kern<<<dim3(g.Lx, R), threads, sm, st>>>(u, gs, g.Lx, tw.y, tw.z, active);
-    PROF_END(KK_ZCONV_C64, R, st);
-    PROF_BEGIN(st);
-    PROF_END(KK_YINV_C64, R, st);
+    PROF_END(KK_SLAB_C64, R, st);
     return cudaGetLastError();
 }
 

@@ -1,0 +1,89 @@
+"""Which passes a complex64 matvec runs, and what launch tracing says of them."""
+import ctypes
+
+import numpy as np
+import pytest
+
+from dda_inputs import random_complex, sphere_grid
+
+pytestmark = pytest.mark.gpu
+
+SEPARATE = {"x_fwd_c64", "y_fwd_c64", "z_conv_c64", "y_inv_c64", "x_inv_c64"}
+SLAB = {"x_fwd_c64", "slab_c64", "x_inv_c64"}
+K1, E1 = np.array([[0.6, 0.0, 0.8]]), np.array([[0.0, 1.0, 0.0]], dtype=complex)
+
+
+@pytest.fixture(scope="module")
+def lib():
+    import paper_1202_3424_gb300 as dda
+    dda.load_library()
+    return dda
+
+
+class Stat(ctypes.Structure):
+    _fields_ = [("name", ctypes.c_char * 24), ("launches", ctypes.c_int64), ("total_ms", ctypes.c_double),
+                ("units", ctypes.c_double)]
+
+
+def _read(lib, ctx, name):
+    """{kind: (launches, ms, units)} by dda_profile_read or dda_profile_kernels."""
+    f = getattr(lib.load_library(), name)
+    f.argtypes = [ctypes.c_void_p, ctypes.POINTER(Stat), ctypes.c_int, ctypes.POINTER(ctypes.c_int)]
+    arr, n = (Stat * 64)(), ctypes.c_int()
+    assert f(ctx.handle, arr, 64, ctypes.byref(n)) == 0
+    return {arr[i].name.decode(): (arr[i].launches, arr[i].total_ms, arr[i].units) for i in range(n.value)}
+
+
+class traced:
+    def __init__(self, lib, ctx):
+        self.lib, self.ctx = lib, ctx
+
+    def __enter__(self):
+        assert self.lib.load_library().dda_profile_enable(self.ctx.handle, 1) == 0
+        return self
+
+    def __exit__(self, *exc):
+        self.kernels = _read(self.lib, self.ctx, "dda_profile_kernels")
+        self.passes = _read(self.lib, self.ctx, "dda_profile_read")
+        self.lib.load_library().dda_profile_enable(self.ctx.handle, 0)
+
+
+def _ctx(lib, grid, m=1.5 + 0.1j, x=1.0):
+    ctx = lib.Context(0)
+    ctx.set_target(grid)
+    ctx.set_materials([m])
+    ctx.prepare_size_parameter(x, lib.Precision.FP32_REFINED)
+    return ctx
+
+
+def _rhs(R):
+    return np.tile(K1, (R, 1)), np.tile(E1, (R, 1))
+
+
+def test_tracing_by_kernel_and_by_pass(lib):
+    """A product through the slab pass and one through the separate passes in
+    one trace: each kernel once under its own name, each pass once per product,
+    the same total time both ways."""
+    ctx = _ctx(lib, sphere_grid(12))
+    k, e = _rhs(2)
+    X = random_complex((2, 3, ctx.info()["ndipoles"]), 3)
+    with traced(lib, ctx) as t:
+        ctx.matvec(2, k, e, X)
+    assert {n: v[0] for n, v in t.kernels.items() if n.endswith("c64")} == dict.fromkeys(SLAB, 1)
+    assert {n: v[0] for n, v in t.passes.items() if n.endswith("c64")} == dict.fromkeys(SEPARATE, 1)
+    slab_ms = t.kernels["slab_c64"][1]
+    assert slab_ms > 0 and t.passes["z_conv_c64"][1] == slab_ms
+    assert t.passes["y_fwd_c64"][1] == t.passes["y_inv_c64"][1] == 0
+    with traced(lib, ctx) as t:
+        ctx.matvec(2, k, e, X)
+        ctx.set_schedule(0)
+        ctx.matvec(2, k, e, X)
+    for name in SEPARATE | SLAB:
+        once = 2 if name in SEPARATE & SLAB else 1
+        assert t.kernels[name][0] == once and t.kernels[name][2] == 2 * once, name
+    for name in SEPARATE:
+        assert t.passes[name][0] == 2 and t.passes[name][2] == 4, name
+    assert "slab_c64" not in t.passes
+    total = [sum(v[1] for v in s.values()) for s in (t.kernels, t.passes)]
+    assert total[0] == pytest.approx(total[1], rel=1e-12)
+    ctx.close()
