@@ -410,8 +410,8 @@ def run_gb300(args):
                "h2d_bytes_per_step": int(k.nbytes + e.nbytes), "d2h_bytes_per_step": int(P_host.nbytes + 72 * R),
                "time_to_solution_ms": t_e2e * 1e3 / args.steps}
 
-    # the matvec schedules the autotuner chose for this RHS count (cached by now)
-    schedule = {"solve": ctx.get_solve_schedule(R),
+    # whether the slab pass ran, and the schedules the autotuner chose for the separate passes
+    schedule = {"slab_pass": ctx.get_slab_pass(R), "solve": ctx.get_solve_schedule(R),
                 "plain_matvec": {"zpass": ctx.get_schedule(R), "xpass_fwd_inv": list(ctx.get_xpass(R)),
                                  "ypass": ctx.get_ypass(R)}}
     roof = roofline(kstats, info, R, w.name)
@@ -816,7 +816,8 @@ def run_matvec_only(args):
     zpass = ctx.get_schedule(R) if args.precision == "fp32" else 0
     xpass = list(ctx.get_xpass(R)) if args.precision == "fp32" else 0
     ypass = ctx.get_ypass(R) if args.precision == "fp32" else 0
-    line = {"mode": "matvec", "workload": w.name, "rhs": R, "precision": args.precision, "zpass": zpass,
+    slab = args.precision == "fp32" and ctx.get_slab_pass(R)
+    line = {"mode": "matvec", "workload": w.name, "rhs": R, "precision": args.precision, "slab_pass": slab, "zpass": zpass,
             "xpass": xpass, "ypass": ypass,
             "ms_per_matvec": ms, "rhs_matvecs_per_s": R / (ms / 1e3), "kernels": kern, "matvec_roofline": mv_roof}
     if args.cufft:

@@ -335,12 +335,16 @@ dda_status dda_grad_qabs(dda_ctx* ctx, dda_precision precision, const double* kh
  *  - the y passes (complex64 only, Ly = 128, 192, 256): 0 the plan of the
  *    staged passes, 1 a radix plan with one exchange fewer (8 x 16,
  *    8 x 8 x 3, 16 x 16).
- * Where no setter below asks for anything, complex64 matvecs whose Ly and Lz
- * are at most 128 run the slab pass instead: the y and z transforms and the
- * product in one kernel over the kx planes, between x passes of its own, without
- * timing anything (anisotropic materials, and a few shapes for which they are
- * faster, keep the passes above).  The queries below still report, and make, the choices the
- * separate passes would run with.
+ * The slab pass stands outside this choice.  It does the y and z transforms and
+ * the product in one kernel over the kx planes, between x passes of its own, and
+ * is built for complex64 where Ly and Lz are at most 128 and the materials are
+ * not anisotropic.  There, products and solves run it without timing anything,
+ * but for a few shapes for which the passes above are faster -- unless
+ * dda_set_slab_pass says otherwise or a setter below has been given anything
+ * but its default, which asks for the passes above.  dda_get_slab_pass says
+ * which; the other queries report, and make, the choices the separate passes
+ * would run with.  To pin the automatic choice, pin both:
+ * dda_set_slab_pass(what dda_get_slab_pass reports), then the schedules.
  * All choices compute the same product; results agree to rounding.  In
  * automatic mode the context times the available choices inside whole
  * matvecs on its own workspace the first time a matvec of a given type and
@@ -351,9 +355,10 @@ dda_status dda_grad_qabs(dda_ctx* ctx, dda_precision precision, const double* kh
  * dda_set_schedule: zpass -1 automatic (the default), 0..4 forces that z
  *   schedule wherever it exists (3 and 4 fall back to 1 and 2 where the
  *   length has one plan, 1..4 to 0 where the register schedules do not exist).
- * dda_set_slice_passes: on -1 automatic, 0 always the separate passes (the
- *   default: measured on GB300 the slice passes are faster only for small
- *   grids outside a solve), 1 the slice passes wherever they are built.
+ * dda_set_slice_passes: on -1 the timed choice between them and the separate
+ *   passes, 0 always the separate passes (the default: measured on GB300 the
+ *   slice passes are faster only for small grids outside a solve), 1 the slice
+ *   passes wherever they are built.
  * dda_set_xpass: xfwd, xinv -1 automatic (the default), 0..3 forces that
  *   x-forward / x-inverse schedule: 0 rows staged through shared memory,
  *   1 + V the warp-local rows with radix plan variant V (Lx = 128, 256, 512:
@@ -371,7 +376,11 @@ dda_status dda_grad_qabs(dda_ctx* ctx, dda_precision precision, const double* kh
  *   plan where it exists.  dda_get_ypass: the y plan of plain matvecs.
  * dda_get_solve_schedule: the z, x-forward, x-inverse and y schedules of the
  *   complex64 matvecs inside a solve of R RHS (those carry the fused BiCGstab
- *   updates and are tuned apart from plain matvecs, with the same candidates). */
+ *   updates and are tuned apart from plain matvecs, with the same candidates).
+ * dda_set_slab_pass: on -1 automatic (the default, above), 0 never, 1 wherever
+ *   it is built, whatever the other setters ask for.  dda_get_slab_pass:
+ *   whether complex64 matvecs of R RHS, plain or in a solve, run it on the
+ *   current target (needs dda_prepare as dda_get_schedule does).               */
 dda_status dda_set_schedule(dda_ctx* ctx, int zpass);
 dda_status dda_set_slice_passes(dda_ctx* ctx, int on);
 dda_status dda_set_xpass(dda_ctx* ctx, int xfwd, int xinv);
@@ -380,6 +389,8 @@ dda_status dda_get_xpass(dda_ctx* ctx, int R, int* xfwd, int* xinv);
 dda_status dda_set_ypass(dda_ctx* ctx, int ypass);
 dda_status dda_get_ypass(dda_ctx* ctx, int R, int* ypass);
 dda_status dda_get_solve_schedule(dda_ctx* ctx, int R, int* zpass, int* xfwd, int* xinv, int* ypass);
+dda_status dda_set_slab_pass(dda_ctx* ctx, int on);
+dda_status dda_get_slab_pass(dda_ctx* ctx, int R, int* on);
 
 /* Launch tracing (the guide's TIMEIT timing switch, per kernel kind rather than
  * per run): when on, every hot-path kernel launch is bracketed by CUDA events

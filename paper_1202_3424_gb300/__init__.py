@@ -27,7 +27,8 @@ __all__ = [
     "dda_incident_field", "dda_grad_qabs", "dda_matvec_device_noalloc", "dda_set_schedule", "dda_get_schedule",
     "dda_nearfield", "dda_nearfield_dims", "dda_set_slice_passes", "dda_scattering_directions", "dda_farfield",
     "dda_angular_averages", "dda_mueller", "dda_set_anisotropic_materials", "dda_set_xpass", "dda_get_xpass",
-    "dda_set_site_materials", "dda_get_solve_schedule", "dda_set_ypass", "dda_get_ypass",
+    "dda_set_site_materials", "dda_get_solve_schedule", "dda_set_ypass", "dda_get_ypass", "dda_set_slab_pass",
+    "dda_get_slab_pass",
 ]
 
 STATUS = {0: "DDA_OK", 1: "DDA_ERR_ARG", 2: "DDA_ERR_CUDA", 3: "DDA_ERR_OOM", 4: "DDA_ERR_SIZE",
@@ -127,6 +128,8 @@ def load_library(build_if_missing: bool = True):
         "dda_set_site_materials": ([vp, _D, ctypes.c_double], ctypes.c_int),
         "dda_get_solve_schedule": ([vp, ctypes.c_int] + [ctypes.POINTER(ctypes.c_int)] * 4, ctypes.c_int),
         "dda_set_ypass": ([vp, ctypes.c_int], ctypes.c_int),
+        "dda_set_slab_pass": ([vp, ctypes.c_int], ctypes.c_int),
+        "dda_get_slab_pass": ([vp, ctypes.c_int, ctypes.POINTER(ctypes.c_int)], ctypes.c_int),
         "dda_get_ypass": ([vp, ctypes.c_int, ctypes.POINTER(ctypes.c_int)], ctypes.c_int),
         "dda_get_xpass": ([vp, ctypes.c_int, ctypes.POINTER(ctypes.c_int), ctypes.POINTER(ctypes.c_int)],
                           ctypes.c_int),
@@ -423,7 +426,7 @@ def dda_set_schedule(ctx, zpass: int):
 
 
 def dda_set_slice_passes(ctx, on: int):
-    """Fused x+y slice passes: -1 timed, 0 never (default), 1 wherever built."""
+    """Fused x+y slice passes: -1 timed against the separate passes, 0 never (default), 1 wherever built."""
     _check(ctx, load_library().dda_set_slice_passes(ctx, int(on)))
 
 
@@ -471,6 +474,18 @@ def dda_get_ypass(ctx, R: int):
     y = ctypes.c_int(-1)
     _check(ctx, load_library().dda_get_ypass(ctx, int(R), ctypes.byref(y)))
     return y.value
+
+
+def dda_set_slab_pass(ctx, on: int):
+    """The complex64 slab pass: -1 by the library's rule (default), 0 never, 1 wherever built."""
+    _check(ctx, load_library().dda_set_slab_pass(ctx, int(on)))
+
+
+def dda_get_slab_pass(ctx, R: int) -> bool:
+    """Whether complex64 matvecs of R RHS run the slab pass."""
+    on = ctypes.c_int(-1)
+    _check(ctx, load_library().dda_get_slab_pass(ctx, int(R), ctypes.byref(on)))
+    return bool(on.value)
 
 
 class Context:
@@ -562,6 +577,12 @@ class Context:
 
     def set_slice_passes(self, on):
         dda_set_slice_passes(self.handle, on)
+
+    def set_slab_pass(self, on):
+        dda_set_slab_pass(self.handle, on)
+
+    def get_slab_pass(self, R):
+        return dda_get_slab_pass(self.handle, R)
 
     def get_schedule(self, R, with_slices=False):
         return dda_get_schedule(self.handle, R, with_slices)

@@ -111,6 +111,7 @@ struct dda_ctx {
     // the BiCGstab solve and on the 128-RHS ellipsoid (1 block of 512 threads
     // per SM), so they are opt-in.
     int force_slices = 0;
+    int force_slab = -1;  // -1 by rule (uses_slab), 0 never, 1 wherever it is built (dda_set_slab_pass)
     int* h_count = nullptr;  // pinned
     // pinned staging of the small tables that go to and from the device, one
     // copy per call in place of one per table (grown on demand, at most
@@ -720,8 +721,10 @@ dda_status pick_schedule(dda_ctx* ctx, int R, bool may_time, PadWork<T>* out, bo
 //   of rounding until single elements of P differ by 1e-3 at tolerance 1e-5
 //   (BiCGstab(2), 65 cycles), and their users compare runs.
 bool uses_slab(const dda_ctx* ctx, int R) {
-    if (ctx->aniso || ctx->force_z >= 0 || ctx->force_xf >= 0 || ctx->force_xi >= 0 || ctx->force_y >= 0 ||
-        ctx->force_slices != 0 || !slab_built(ctx->g))
+    if (ctx->aniso || !slab_built(ctx->g)) return false;
+    if (ctx->force_slab >= 0) return ctx->force_slab == 1;
+    // (slices -1 asks for the timed choice among the separate passes)
+    if (ctx->force_z >= 0 || ctx->force_xf >= 0 || ctx->force_xi >= 0 || ctx->force_y >= 0 || ctx->force_slices != 0)
         return false;
     const Geom& g = ctx->g;
     const int64_t slabs = (int64_t)g.Lx * R, points = (int64_t)g.Ly * g.Lz;
@@ -2489,6 +2492,26 @@ dda_status dda_set_slice_passes(dda_ctx* ctx, int on) {
         cudaGraphExecDestroy(ctx->graph.exec);
         ctx->graph.exec = nullptr;
     }
+    return DDA_OK;
+}
+
+dda_status dda_set_slab_pass(dda_ctx* ctx, int on) {
+    if (!ctx) return DDA_ERR_ARG;
+    if (on < -1 || on > 1) return ctx->fail(DDA_ERR_ARG, "slab pass: -1, 0 or 1 (got %d)", on);
+    ctx->force_slab = on;
+    if (ctx->graph.exec) {
+        cudaGraphExecDestroy(ctx->graph.exec);
+        ctx->graph.exec = nullptr;
+    }
+    return DDA_OK;
+}
+
+dda_status dda_get_slab_pass(dda_ctx* ctx, int R, int* on) {
+    if (!ctx || !on) return DDA_ERR_ARG;
+    if (R <= 0) return ctx->fail(DDA_ERR_ARG, "R must be > 0");
+    if (!ctx->prepared || !ctx->has32)
+        return ctx->fail(DDA_ERR_ARG, "dda_prepare with a complex64-capable precision has not been called");
+    *on = uses_slab(ctx, matvec_chunk<float>(ctx, R));
     return DDA_OK;
 }
 

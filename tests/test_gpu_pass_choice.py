@@ -87,3 +87,66 @@ def test_tracing_by_kernel_and_by_pass(lib):
     total = [sum(v[1] for v in s.values()) for s in (t.kernels, t.passes)]
     assert total[0] == pytest.approx(total[1], rel=1e-12)
     ctx.close()
+
+
+def _runs_slab(lib, ctx, R):
+    """Whether the kernels of a product of R right-hand sides are the slab pass's; the query has to agree."""
+    k, e = _rhs(R)
+    X = random_complex((R, 3, ctx.info()["ndipoles"]), 3)
+    with traced(lib, ctx) as t:
+        ctx.matvec(2, k, e, X)
+    ran = {n for n in t.kernels if n.endswith("c64")}
+    assert ran in (SLAB, SEPARATE)
+    assert ctx.get_slab_pass(R) == (ran == SLAB)
+    return ran == SLAB
+
+
+def test_slab_pass_is_asked_for_refused_and_queried(lib):
+    """The setter against every other setter, and back to the rule; what the
+    query reports pins the automatic choice, bit for bit."""
+    ctx = _ctx(lib, sphere_grid(12))
+    k, e = _rhs(2)
+    X = random_complex((2, 3, ctx.info()["ndipoles"]), 3)
+    assert _runs_slab(lib, ctx, 2)
+    auto = ctx.matvec(2, k, e, X)
+    ctx.set_slab_pass(0)
+    assert not _runs_slab(lib, ctx, 2)
+    ctx.set_slab_pass(-1)
+    for setter, value, default in ((ctx.set_schedule, 0, -1), (ctx.set_xpass, 0, -1), (ctx.set_ypass, 0, -1),
+                                   (ctx.set_slice_passes, -1, 0)):
+        setter(value)
+        assert not ctx.get_slab_pass(2)
+        ctx.set_slab_pass(1)
+        assert _runs_slab(lib, ctx, 2)
+        ctx.set_slab_pass(-1)
+        setter(default)
+        assert ctx.get_slab_pass(2)
+    # pinned, with the separate passes' schedules pinned after it
+    ctx.set_slab_pass(ctx.get_slab_pass(2))
+    ctx.set_schedule(ctx.get_schedule(2))
+    ctx.set_xpass(ctx.get_xpass(2))
+    ctx.set_ypass(ctx.get_ypass(2))
+    assert np.array_equal(ctx.matvec(2, k, e, X), auto)
+    for bad in (-2, 2):
+        with pytest.raises(lib.DdaError):
+            ctx.set_slab_pass(bad)
+    ctx.close()
+
+
+def test_slab_pass_where_it_is_not_built(lib):
+    """Asked for, it still leaves long axes, tilted crystals and the other
+    arithmetics to the separate passes."""
+    ctx = _ctx(lib, np.ones((2, 70, 2), np.uint8))     # Ly = 192
+    ctx.set_slab_pass(1)
+    assert not _runs_slab(lib, ctx, 2)
+    ctx.set_target(sphere_grid(12))
+    ctx.set_anisotropic_materials([[1.5, 1.6, 1.4]], [(0.4, 1.1, -0.6)])
+    ctx.prepare_size_parameter(1.0, lib.Precision.FP32_REFINED)
+    assert not _runs_slab(lib, ctx, 2)
+    ctx.set_materials([1.5 + 0.1j])
+    with pytest.raises(lib.DdaError):
+        ctx.get_slab_pass(2)                            # not prepared
+    ctx.prepare_size_parameter(1.0, lib.Precision.FP64)
+    with pytest.raises(lib.DdaError):
+        ctx.get_slab_pass(2)                            # no complex64 tensor
+    ctx.close()
