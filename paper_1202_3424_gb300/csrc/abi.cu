@@ -1106,12 +1106,13 @@ dda_status solve_core(dda_ctx* ctx, int R, const dda_opts& o, bool refine, bool 
     const int max_outer = refine ? (o.max_outer > 0 ? o.max_outer : 8) : 1;
     const double floor_tol = (sizeof(T) == 4) ? (o.inner_tol > 0 ? o.inner_tol : 2e-6) : 1e-15;
     // Where an inner solve stops, as a part of what its RHS still needs.  The
-    // slab pass rounds in another order than the separate passes, which BiCGstab
-    // turns into another last iterate: stopped at half the tolerance, single
-    // results came out up to 1.7 times further from the exact solution than the
-    // separate passes' (64^3 sphere; the mean was the same).  A third costs about
-    // one iteration in thirty and keeps them from it.
-    const double share = (sizeof(T) == 4 && uses_slab(ctx, matvec_chunk<T>(ctx, R))) ? 1.0 / 3.0 : 0.5;
+    // last iterate's error can be twice its residual and more, so a complex64
+    // solve stopped at half the tolerance can miss the solution by more than the
+    // tolerance; a third keeps it within.  64^3 sphere, 12 directions, tolerance
+    // 1e-5, largest error 1.1e-5 -> 5.6e-6 through the separate passes (5.0e-6
+    // through the slab pass), for one product in sixty (a strongly absorbing brick
+    // with BiCGstab(2): 2 % of its time).
+    const double share = sizeof(T) == 4 ? 1.0 / 3.0 : 0.5;
     Inner<T> in = InnerSlots<T>::get(ctx);
     for (int it = 0; it < max_outer; ++it) {
         int nact = 0;

@@ -150,3 +150,23 @@ def test_slab_pass_where_it_is_not_built(lib):
     with pytest.raises(lib.DdaError):
         ctx.get_slab_pass(2)                            # no complex64 tensor
     ctx.close()
+
+
+def test_refined_solves_stop_alike_on_either_passes(lib):
+    """Inner solves stop at a third of the tolerance, whichever passes run: the
+    true residual exceeds that by the drift of the FP32 recurrence alone (some
+    sixty products, 2^-24 each, of a solution of the incident field's size: 4e-6)."""
+    ctx = _ctx(lib, sphere_grid(24), 1.5 + 0.02j, 3.0)
+    rng = np.random.default_rng(2)
+    k = rng.standard_normal((16, 3))
+    k /= np.linalg.norm(k, axis=1)[:, None]
+    e = np.cross(k, [0.0, 0.0, 1.0])
+    e = (e / np.linalg.norm(e, axis=1)[:, None]).astype(complex)
+    tol = 1e-4
+    for on in (0, 1):
+        ctx.set_slab_pass(on)
+        for solver in ("bicgstab", "bicgstab2", "qmr"):
+            res, _, st = ctx.solve(lib.Precision.FP32_REFINED, k, e, want_P=False, tol=tol, maxit=400, solver=solver)
+            assert st == 0
+            assert max(r["resid_rel"] for r in res) <= tol / 3 + 4e-6, (on, solver)
+    ctx.close()
