@@ -411,7 +411,7 @@ def run_gb300(args):
                "time_to_solution_ms": t_e2e * 1e3 / args.steps}
 
     # whether the slab pass ran, and the schedules the autotuner chose for the separate passes
-    schedule = {"slab_pass": ctx.get_slab_pass(R), "solve": ctx.get_solve_schedule(R),
+    schedule = {"slab_pass": ctx.get_slab_pass(R, solve=True), "solve": ctx.get_solve_schedule(R),
                 "plain_matvec": {"zpass": ctx.get_schedule(R), "xpass_fwd_inv": list(ctx.get_xpass(R)),
                                  "ypass": ctx.get_ypass(R)}}
     roof = roofline(kstats, info, R, w.name)

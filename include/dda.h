@@ -343,8 +343,8 @@ dda_status dda_grad_qabs(dda_ctx* ctx, dda_precision precision, const double* kh
  * dda_set_slab_pass says otherwise or a setter below has been given anything
  * but its default, which asks for the passes above.  dda_get_slab_pass says
  * which; the other queries report, and make, the choices the separate passes
- * would run with.  To pin the automatic choice, pin both:
- * dda_set_slab_pass(what dda_get_slab_pass reports), then the schedules.
+ * would run with.  To pin the automatic choice of products (or of solves), pin
+ * both: dda_set_slab_pass(what dda_get_slab_pass reports), then the schedules.
  * All choices compute the same product; results agree to rounding.  In
  * automatic mode the context times the available choices inside whole
  * matvecs on its own workspace the first time a matvec of a given type and
@@ -379,8 +379,8 @@ dda_status dda_grad_qabs(dda_ctx* ctx, dda_precision precision, const double* kh
  *   updates and are tuned apart from plain matvecs, with the same candidates).
  * dda_set_slab_pass: on -1 automatic (the default, above), 0 never, 1 wherever
  *   it is built, whatever the other setters ask for.  dda_get_slab_pass:
- *   whether complex64 matvecs of R RHS, plain or in a solve, run it on the
- *   current target (needs dda_prepare as dda_get_schedule does).               */
+ *   whether complex64 matvecs of R RHS run it on the current target, plain
+ *   ones and those in a solve (needs dda_prepare as dda_get_schedule does).    */
 dda_status dda_set_schedule(dda_ctx* ctx, int zpass);
 dda_status dda_set_slice_passes(dda_ctx* ctx, int on);
 dda_status dda_set_xpass(dda_ctx* ctx, int xfwd, int xinv);
@@ -390,7 +390,7 @@ dda_status dda_set_ypass(dda_ctx* ctx, int ypass);
 dda_status dda_get_ypass(dda_ctx* ctx, int R, int* ypass);
 dda_status dda_get_solve_schedule(dda_ctx* ctx, int R, int* zpass, int* xfwd, int* xinv, int* ypass);
 dda_status dda_set_slab_pass(dda_ctx* ctx, int on);
-dda_status dda_get_slab_pass(dda_ctx* ctx, int R, int* on);
+dda_status dda_get_slab_pass(dda_ctx* ctx, int R, int* plain, int* solve);
 
 /* Launch tracing (the guide's TIMEIT timing switch, per kernel kind rather than
  * per run): when on, every hot-path kernel launch is bracketed by CUDA events

@@ -129,7 +129,8 @@ def load_library(build_if_missing: bool = True):
         "dda_get_solve_schedule": ([vp, ctypes.c_int] + [ctypes.POINTER(ctypes.c_int)] * 4, ctypes.c_int),
         "dda_set_ypass": ([vp, ctypes.c_int], ctypes.c_int),
         "dda_set_slab_pass": ([vp, ctypes.c_int], ctypes.c_int),
-        "dda_get_slab_pass": ([vp, ctypes.c_int, ctypes.POINTER(ctypes.c_int)], ctypes.c_int),
+        "dda_get_slab_pass": ([vp, ctypes.c_int, ctypes.POINTER(ctypes.c_int), ctypes.POINTER(ctypes.c_int)],
+                              ctypes.c_int),
         "dda_get_ypass": ([vp, ctypes.c_int, ctypes.POINTER(ctypes.c_int)], ctypes.c_int),
         "dda_get_xpass": ([vp, ctypes.c_int, ctypes.POINTER(ctypes.c_int), ctypes.POINTER(ctypes.c_int)],
                           ctypes.c_int),
@@ -481,11 +482,11 @@ def dda_set_slab_pass(ctx, on: int):
     _check(ctx, load_library().dda_set_slab_pass(ctx, int(on)))
 
 
-def dda_get_slab_pass(ctx, R: int) -> bool:
-    """Whether complex64 matvecs of R RHS run the slab pass."""
-    on = ctypes.c_int(-1)
-    _check(ctx, load_library().dda_get_slab_pass(ctx, int(R), ctypes.byref(on)))
-    return bool(on.value)
+def dda_get_slab_pass(ctx, R: int, solve: bool = False) -> bool:
+    """Whether complex64 matvecs of R RHS run the slab pass: plain ones, or those in a solve."""
+    p, s = ctypes.c_int(-1), ctypes.c_int(-1)
+    _check(ctx, load_library().dda_get_slab_pass(ctx, int(R), ctypes.byref(p), ctypes.byref(s)))
+    return bool(s.value if solve else p.value)
 
 
 class Context:
@@ -581,8 +582,8 @@ class Context:
     def set_slab_pass(self, on):
         dda_set_slab_pass(self.handle, on)
 
-    def get_slab_pass(self, R):
-        return dda_get_slab_pass(self.handle, R)
+    def get_slab_pass(self, R, solve=False):
+        return dda_get_slab_pass(self.handle, R, solve)
 
     def get_schedule(self, R, with_slices=False):
         return dda_get_schedule(self.handle, R, with_slices)

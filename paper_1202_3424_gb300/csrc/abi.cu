@@ -707,20 +707,24 @@ dda_status pick_schedule(dda_ctx* ctx, int R, bool may_time, PadWork<T>* out, bo
     return DDA_OK;
 }
 
-// Whether complex64 matvecs of R right-hand sides run the slab pass (slab.cuh):
-// where it is built and no setter asks for a schedule of the separate passes,
-// which it replaces.  Whole products, separate passes / slab: 96x64x32 ellipsoid,
-// 32 RHS 931 / 763 us; 64^3 sphere, 2 RHS 109 / 90 us; 48^3, 4 RHS 134 / 108 us; over
-// padded lengths 32..128 (x to 256) and 1, 3 and 12 RHS 1.0-1.45 times faster, but
-// for these, which keep the separate passes:
+// Whether complex64 matvecs of R right-hand sides run the slab pass (slab.cuh),
+// in a product of its own or in a solve: where it is built and no setter asks
+// for a schedule of the separate passes, which it replaces.  (Its x-inverse is
+// not instantiated for the tensors of anisotropic materials.)  Products,
+// separate passes / slab: 96x64x32 ellipsoid, 32 RHS 931 / 763 us; 64^3 sphere,
+// 2 RHS 109 / 90 us; 48^3, 4 RHS 134 / 108 us.  These keep the separate passes:
 //   many long, thin slabs, whose x passes, faster row by row, are most of the
-//   work: 256x48x32 padded, 12 RHS 119 / 125 us; 128x32x48 97 / 103 us;
-//   a few large slabs, which occupy a fifth of the SMs: 32x128x96 padded, 1 RHS
-//   54 / 58 us;
-//   anisotropic materials: solves of strongly absorbing crystals amplify a change
-//   of rounding until single elements of P differ by 1e-3 at tolerance 1e-5
-//   (BiCGstab(2), 65 cycles), and their users compare runs.
-bool uses_slab(const dda_ctx* ctx, int R) {
+//   work: padded 512x16x48, 12 RHS 159 / 228 us; 256x16x48 99 / 128 us; 128x32x48
+//   97 / 104 us;
+//   a few large slabs, which occupy a third of the SMs or less: 32x128x96, 1 RHS
+//   53 / 59 us, and in solves, whose replayed graphs take most of the cost of
+//   two more launches away, earlier: per product 48x96x96 67 / 74 us, 32x96x48
+//   36 / 38 us (as products of their own 1.05 and 1.08 times faster).
+// Over all 1080 shapes of padded lengths 16..512 by 16..128 by 16..128 with 1, 3
+// and 12 RHS the slab pass is 0.99..1.8 times as fast where the rule takes it
+// (median 1.21), and 0.70..1.29 where it does not: thin slabs differ among
+// themselves, and the line keeps every shape from losing.
+bool uses_slab(const dda_ctx* ctx, int R, bool in_solve) {
     if (ctx->aniso || !slab_built(ctx->g)) return false;
     if (ctx->force_slab >= 0) return ctx->force_slab == 1;
     // (slices -1 asks for the timed choice among the separate passes)
@@ -730,14 +734,15 @@ bool uses_slab(const dda_ctx* ctx, int R) {
     const int64_t slabs = (int64_t)g.Lx * R, points = (int64_t)g.Ly * g.Lz;
     if (slabs >= 1024 && g.Lx >= 128 && points <= 12 * g.Lx) return false;
     if (slabs < 48 && points >= 64 * 96) return false;
+    if (in_solve && R == 1 && slabs <= 48 && points >= (slabs < 48 ? 48 * 96 : 96 * 96)) return false;
     return true;
 }
 // The passes of a matvec: the slab pass, or pick_schedule's choice.
 template <typename T>
-dda_status choose_passes(dda_ctx* ctx, int R, bool may_time, PadWork<T>* out, bool fused = false) {
+dda_status choose_passes(dda_ctx* ctx, int R, bool may_time, PadWork<T>* out, bool in_solve, bool fused = false) {
     out->slab = nullptr;
     if constexpr (std::is_same<T, float>::value) {
-        if (uses_slab(ctx, R)) {
+        if (uses_slab(ctx, R, in_solve)) {
             out->slab = static_cast<const float4*>(ctx->m_ghslab.p);
             return DDA_OK;
         }
@@ -745,7 +750,8 @@ dda_status choose_passes(dda_ctx* ctx, int R, bool may_time, PadWork<T>* out, bo
     return pick_schedule<T>(ctx, R, may_time, out, fused);
 }
 
-// y = A x over R RHS in chunks (workspace from ensure_pad<T>).
+// y = A x over R RHS in chunks (workspace from ensure_pad<T>).  active: the
+// flags of a solve's RHS, or null for a product of its own.
 template <typename T>
 dda_status run_matvec(dda_ctx* ctx, int R, const cx<T>* x, cx<T>* y, const int* active) {
     const int rc = matvec_chunk<T>(ctx, R);
@@ -756,7 +762,7 @@ dda_status run_matvec(dda_ctx* ctx, int R, const cx<T>* x, cx<T>* y, const int* 
     dda_status zs;
     for (int r0 = 0; r0 < R; r0 += rc) {
         const int rn = std::min(rc, R - r0);
-        if ((zs = choose_passes<T>(ctx, rn, true, &w)) != DDA_OK) return zs;
+        if ((zs = choose_passes<T>(ctx, rn, true, &w, active != nullptr)) != DDA_OK) return zs;
         CU(launch_matvec<T>(ctx->g, rn, x + (int64_t)r0 * n, y + (int64_t)r0 * n, w, ctx->tg,
                             beta_of<T>(ctx) + (int64_t)r0 * BS, BS, ghat_of<T>(ctx), tw_of<T>(ctx),
                             active ? active + r0 : nullptr, ctx->stream));
@@ -820,7 +826,7 @@ dda_status run_matvec_fused(dda_ctx* ctx, int R, int mode, cx<T>* x, cx<T>* y, c
     for (int r0 = 0; r0 < R; r0 += rc) {
         const int rn = std::min(rc, R - r0);
         const int64_t o = (int64_t)r0 * n;
-        if ((zs = choose_passes<T>(ctx, rn, true, &w, true)) != DDA_OK) return zs;
+        if ((zs = choose_passes<T>(ctx, rn, true, &w, true, true)) != DDA_OK) return zs;
         FusedKrylov<T> fk;
         fk.mode = mode;
         fk.r = r + o;
@@ -1403,7 +1409,7 @@ dda_status matvec_noalloc(dda_ctx* ctx, int R, const std::vector<double>& k, con
     w.beta_tensor = ctx->aniso;
     CU(cudaMemcpyAsync(d_beta, beta.data(), beta.size() * sizeof(C), cudaMemcpyHostToDevice, ctx->stream));
     dda_status zs;
-    if ((zs = choose_passes<T>(ctx, R, false, &w)) != DDA_OK) return zs;  // no timing here
+    if ((zs = choose_passes<T>(ctx, R, false, &w, false)) != DDA_OK) return zs;  // no timing here
     CU(launch_matvec<T>(ctx->g, R, static_cast<const C*>(x_dev), static_cast<C*>(y_dev), w, ctx->tg, d_beta, BS,
                         ghat_of<T>(ctx), tw_of<T>(ctx), nullptr, ctx->stream));
     CU(cudaStreamSynchronize(ctx->stream));
@@ -2507,12 +2513,13 @@ dda_status dda_set_slab_pass(dda_ctx* ctx, int on) {
     return DDA_OK;
 }
 
-dda_status dda_get_slab_pass(dda_ctx* ctx, int R, int* on) {
-    if (!ctx || !on) return DDA_ERR_ARG;
+dda_status dda_get_slab_pass(dda_ctx* ctx, int R, int* plain, int* solve) {
+    if (!ctx || !plain || !solve) return DDA_ERR_ARG;
     if (R <= 0) return ctx->fail(DDA_ERR_ARG, "R must be > 0");
     if (!ctx->prepared || !ctx->has32)
         return ctx->fail(DDA_ERR_ARG, "dda_prepare with a complex64-capable precision has not been called");
-    *on = uses_slab(ctx, matvec_chunk<float>(ctx, R));
+    *plain = uses_slab(ctx, matvec_chunk<float>(ctx, R), false);
+    *solve = uses_slab(ctx, matvec_chunk<float>(ctx, R), true);
     return DDA_OK;
 }
 

@@ -170,3 +170,43 @@ def test_refined_solves_stop_alike_on_either_passes(lib):
             assert st == 0
             assert max(r["resid_rel"] for r in res) <= tol / 3 + 4e-6, (on, solver)
     ctx.close()
+
+
+# (lattice, R, plain products, solves): both sides of every line of the rule
+RULE = [
+    ((16, 24, 24), 1, True, True),       # 32 slabs of 48 x 48
+    ((16, 48, 24), 1, True, False),      # of 96 x 48: a solve's lost 5 %
+    ((16, 48, 24), 2, True, True),
+    ((16, 64, 48), 1, False, False),     # of 128 x 96
+    ((16, 64, 48), 2, True, True),
+    ((24, 48, 48), 1, True, False),      # 48 slabs of 96 x 96: a solve's lost 10 %
+    ((24, 48, 24), 1, True, True),
+    ((24, 48, 48), 2, True, True),
+    ((64, 16, 24), 8, False, False),     # 1024 slabs of 32 x 48
+    ((64, 16, 24), 7, True, True),
+    ((64, 24, 24), 8, True, True),
+    ((48, 16, 16), 12, True, True),      # 96 points along x
+]
+
+
+@pytest.mark.parametrize("n,R,plain,solve", RULE, ids=["x".join(map(str, c[0])) + f"_R{c[1]}" for c in RULE])
+def test_rule_decides_which_passes_run(lib, n, R, plain, solve):
+    """The kernels that run are those the rule names, in a product and in a
+    solve, and agree with the other passes' to the complex64 tolerance."""
+    grid = np.zeros(n[::-1], np.uint8)
+    grid[:3, :3, :3] = grid[-3:, -3:, -3:] = 1
+    ctx = _ctx(lib, grid, 1.5 + 0.05j)
+    assert (ctx.get_slab_pass(R), ctx.get_slab_pass(R, solve=True)) == (plain, solve)
+    assert _runs_slab(lib, ctx, R) == plain
+    k, e = _rhs(R)
+    X = random_complex((R, 3, ctx.info()["ndipoles"]), 3)
+    auto = ctx.matvec(2, k, e, X)
+    for solver in ("bicgstab", "bicgstab2", "qmr"):
+        with traced(lib, ctx) as t:
+            _, P, st = ctx.solve(lib.Precision.FP32_REFINED, k, e, tol=1e-6, solver=solver)
+        assert st == 0
+        assert ("slab_c64" in t.kernels, "z_conv_c64" in t.kernels) == (solve, not solve)
+    ctx.set_slab_pass(int(not plain))
+    other = ctx.matvec(2, k, e, X)
+    assert np.abs(auto - other).max() < 1e-5 * np.abs(other).max()
+    ctx.close()
