@@ -718,7 +718,7 @@ dda_status pick_schedule(dda_ctx* ctx, int R, bool may_time, PadWork<T>* out, bo
 //   97 / 104 us;
 //   a few large slabs, which occupy a third of the SMs or less: 32x128x96, 1 RHS
 //   53 / 59 us, and in solves, whose replayed graphs take most of the cost of
-//   two more launches away, earlier: per product 48x96x96 67 / 74 us, 32x96x48
+//   two more launches away, earlier: per product 48x96x96 45 / 50 us, 32x96x48
 //   36 / 38 us (as products of their own 1.05 and 1.08 times faster).
 // Over all 1080 shapes of padded lengths 16..512 by 16..128 by 16..128 with 1, 3
 // and 12 RHS the slab pass is 0.99..1.8 times as fast where the rule takes it
