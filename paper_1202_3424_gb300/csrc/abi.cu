@@ -92,7 +92,8 @@ struct dda_ctx {
     bool prepared = false, has32 = false;
     double kd = 0.0, aeff_lat = 0.0;
     DevMem m_gh64, m_gh32, m_tw64[3], m_tw32[3];
-    DevMem m_ghslab;           // the slab pass's copy (slab.cuh), where that pass is built
+    DevMem m_ghslab;           // the slab pass's copy (slab.cuh), where that pass can run
+    bool has_slab = false;     // m_ghslab holds the prepared wavelength's
     DevMem m_ghdf, m_twdf[3];  // double-float copies for the refinement residual
 
     // workspace
@@ -707,6 +708,33 @@ dda_status pick_schedule(dda_ctx* ctx, int R, bool may_time, PadWork<T>* out, bo
     return DDA_OK;
 }
 
+// Whether the setters and the target leave a place for the slab pass at all.
+bool slab_wanted(const dda_ctx* ctx) {
+    if (ctx->aniso || ctx->force_slab == 0 || !slab_built(ctx->g)) return false;
+    if (ctx->force_slab == 1) return true;
+    // (slices -1 asks for the timed choice among the separate passes)
+    return ctx->force_z < 0 && ctx->force_xf < 0 && ctx->force_xi < 0 && ctx->force_y < 0 && ctx->force_slices == 0;
+}
+// The slab pass's copy of the Green tensor, nearly twice the octant's size, is
+// made by dda_prepare or, where a setter has made a place for it since, at the
+// first call that runs it and may allocate.  Where there is no memory for it,
+// the separate passes serve.
+dda_status ensure_slab(dda_ctx* ctx) {
+    if (ctx->has_slab) return DDA_OK;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    CU(cudaStreamIsCapturing(ctx->stream, &cs));
+    if (cs != cudaStreamCaptureStatusNone) return DDA_OK;
+    const std::string err = ctx->err;
+    const dda_status s = ensure(ctx, ctx->m_ghslab, slab_green_size(ctx->g) * sizeof(float4));
+    if (s == DDA_ERR_OOM) {
+        ctx->err = err;
+        return DDA_OK;
+    }
+    if (s != DDA_OK) return s;
+    CU(launch_slab_green(ctx->g, (const double2*)ctx->m_gh64.p, (float4*)ctx->m_ghslab.p, ctx->stream));
+    ctx->has_slab = true;
+    return DDA_OK;
+}
 // Whether complex64 matvecs of R right-hand sides run the slab pass (slab.cuh),
 // in a product of its own or in a solve: where it is built and no setter asks
 // for a schedule of the separate passes, which it replaces.  (Its x-inverse is
@@ -725,11 +753,8 @@ dda_status pick_schedule(dda_ctx* ctx, int R, bool may_time, PadWork<T>* out, bo
 // (median 1.21), and 0.70..1.29 where it does not: thin slabs differ among
 // themselves, and the line keeps every shape from losing.
 bool uses_slab(const dda_ctx* ctx, int R, bool in_solve) {
-    if (ctx->aniso || !slab_built(ctx->g)) return false;
-    if (ctx->force_slab >= 0) return ctx->force_slab == 1;
-    // (slices -1 asks for the timed choice among the separate passes)
-    if (ctx->force_z >= 0 || ctx->force_xf >= 0 || ctx->force_xi >= 0 || ctx->force_y >= 0 || ctx->force_slices != 0)
-        return false;
+    if (!slab_wanted(ctx)) return false;
+    if (ctx->force_slab == 1) return true;
     const Geom& g = ctx->g;
     const int64_t slabs = (int64_t)g.Lx * R, points = (int64_t)g.Ly * g.Lz;
     if (slabs >= 1024 && g.Lx >= 128 && points <= 12 * g.Lx) return false;
@@ -742,7 +767,10 @@ template <typename T>
 dda_status choose_passes(dda_ctx* ctx, int R, bool may_time, PadWork<T>* out, bool in_solve, bool fused = false) {
     out->slab = nullptr;
     if constexpr (std::is_same<T, float>::value) {
-        if (uses_slab(ctx, R, in_solve)) {
+        dda_status s;
+        const bool slab = uses_slab(ctx, R, in_solve);
+        if (slab && may_time && (s = ensure_slab(ctx)) != DDA_OK) return s;
+        if (slab && ctx->has_slab) {
             out->slab = static_cast<const float4*>(ctx->m_ghslab.p);
             return DDA_OK;
         }
@@ -1750,16 +1778,13 @@ dda_status dda_prepare(dda_ctx* ctx, double lambda_vac, double aeff, dda_precisi
     if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
     if (sb > kKeepMax) free_mem(ctx->pool[S_GREEN]);
     if (e != cudaSuccess) return ctx->cuda_fail(e, "Green tensor FFT");
-    ctx->has32 = false;
+    ctx->has32 = ctx->has_slab = false;
     if (precision != DDA_FP64) {
         if ((s = ensure(ctx, ctx->m_gh32, oct * sizeof(float2))) != DDA_OK) return s;
         CU(launch_convert_c128_to_c64((const double2*)ctx->m_gh64.p, (float2*)ctx->m_gh32.p, oct, ctx->stream));
         if ((s = ensure(ctx, ctx->m_ghdf, oct * sizeof(cdfl))) != DDA_OK) return s;
         CU(launch_convert_c128_to_df((const double2*)ctx->m_gh64.p, (cdfl*)ctx->m_ghdf.p, oct, ctx->stream));
-        if (slab_built(g)) {
-            if ((s = ensure(ctx, ctx->m_ghslab, slab_green_size(g) * sizeof(float4))) != DDA_OK) return s;
-            CU(launch_slab_green(g, (const double2*)ctx->m_gh64.p, (float4*)ctx->m_ghslab.p, ctx->stream));
-        }
+        if (slab_wanted(ctx) && (s = ensure_slab(ctx)) != DDA_OK) return s;
         CU(sync_collect(ctx));
         ctx->has32 = true;
     }
@@ -2518,9 +2543,14 @@ dda_status dda_get_slab_pass(dda_ctx* ctx, int R, int* plain, int* solve) {
     if (R <= 0) return ctx->fail(DDA_ERR_ARG, "R must be > 0");
     if (!ctx->prepared || !ctx->has32)
         return ctx->fail(DDA_ERR_ARG, "dda_prepare with a complex64-capable precision has not been called");
-    *plain = uses_slab(ctx, matvec_chunk<float>(ctx, R), false);
-    *solve = uses_slab(ctx, matvec_chunk<float>(ctx, R), true);
-    return DDA_OK;
+    const int rc = matvec_chunk<float>(ctx, R);
+    *plain = uses_slab(ctx, rc, false);
+    *solve = uses_slab(ctx, rc, true);
+    if (!*plain && !*solve) return DDA_OK;
+    cudaSetDevice(ctx->device);
+    const dda_status s = ensure_slab(ctx);
+    if (!ctx->has_slab) *plain = *solve = 0;
+    return s;
 }
 
 dda_status dda_get_schedule(dda_ctx* ctx, int R, int* zpass, int* slices) {

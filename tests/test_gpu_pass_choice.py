@@ -210,3 +210,74 @@ def test_rule_decides_which_passes_run(lib, n, R, plain, solve):
     other = ctx.matvec(2, k, e, X)
     assert np.abs(auto - other).max() < 1e-5 * np.abs(other).max()
     ctx.close()
+
+
+def _device_bytes(f):
+    import torch
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    f()
+    torch.cuda.synchronize()
+    return before - torch.cuda.mem_get_info()[0]
+
+
+def test_slab_tensor_is_kept_only_where_it_can_be_used(lib):
+    """The slab pass's copy of the Green tensor (26 MB for a 64^3 lattice) is
+    made for targets and schedules that can take the pass, and at the first
+    product where a setter makes a place for it later."""
+    grid = sphere_grid(64)
+    size = (65 * 64 * 128 * 3 + 65 * 128 * 3) * 16
+
+    def prepared(aniso, schedule):
+        ctx = lib.Context(0)
+        ctx.set_target(grid)
+        if aniso:
+            ctx.set_anisotropic_materials([[1.5, 1.6, 1.4]], [(0.4, 1.1, -0.6)])
+        else:
+            ctx.set_materials([1.5 + 0.1j])
+        ctx.set_schedule(schedule)
+        return ctx, _device_bytes(lambda: ctx.prepare_size_parameter(1.0, lib.Precision.FP32_REFINED))
+
+    prepared(False, -1)[0].close()                       # (modules loaded)
+    (iso, b_iso), (crystal, b_crystal), (forced, b_forced) = (prepared(*a) for a in ((False, -1), (True, -1), (False, 0)))
+    slack = 4 << 20                                      # the allocator's granularity
+    assert b_iso - b_crystal > size - slack and b_iso - b_forced > size - slack
+    k, e = _rhs(1)
+    X = random_complex((1, 3, iso.info()["ndipoles"]), 3)
+    before = forced.matvec(2, k, e, X)
+    forced.set_schedule(-1)
+    assert _runs_slab(lib, forced, 1)
+    after = forced.matvec(2, k, e, X)
+    assert np.array_equal(after, iso.matvec(2, k, e, X)) and not np.array_equal(after, before)
+    # another wavelength: the copy is the new one's
+    for ctx in (forced, iso):
+        ctx.prepare_size_parameter(2.0, lib.Precision.FP32_REFINED)
+    forced.set_slab_pass(0)
+    want = forced.matvec(2, k, e, X)
+    assert np.abs(iso.matvec(2, k, e, X) - want).max() < 1e-5 * np.abs(want).max()
+    for ctx in (iso, crystal, forced):
+        ctx.close()
+
+
+def test_no_allocation_product_after_a_schedule_was_forced(lib):
+    """A product that may not allocate takes the slab pass once its copy of the
+    tensor is there, and the separate passes until then."""
+    import torch
+    ctx = lib.Context(0)
+    ctx.set_target(sphere_grid(12))
+    ctx.set_materials([1.5 + 0.1j])
+    ctx.set_schedule(0)
+    ctx.prepare_size_parameter(1.0, lib.Precision.FP32_REFINED)
+    ctx.set_schedule(-1)
+    k, e = _rhs(2)
+    x = torch.from_numpy(random_complex((2, 3, ctx.info()["ndipoles"]), 3).astype(np.complex64)).cuda()
+    y0, y1, slab = (torch.empty_like(x) for _ in range(3))
+    torch.cuda.synchronize()
+    lib.dda_matvec_device_noalloc(ctx.handle, 2, k, e, x, y0)
+    assert ctx.get_slab_pass(2)                         # makes the copy
+    lib.dda_matvec_device_noalloc(ctx.handle, 2, k, e, x, y1)
+    lib.dda_matvec_device(ctx.handle, 2, k, e, x, slab)
+    y0, y1, slab = (y.cpu().numpy() for y in (y0, y1, slab))
+    assert np.array_equal(y1, slab) and not np.array_equal(y0, slab)
+    assert np.abs(y0 - y1).max() < 1e-5 * np.abs(y0).max()
+    ctx.close()
