@@ -40,8 +40,12 @@
  *    normalized, transverse to khat.
  *  - Ownership: the caller owns every host buffer it passes (read during the
  *    call only; never retained).  The context owns all device memory it
- *    allocates.  Device-pointer variants (suffix _device) read/write
- *    caller-owned device buffers and run on the context's stream.
+ *    allocates, and keeps it for later calls: the solver's workspace at its
+ *    largest size so far, and the scratch of dda_prepare and of the near- and
+ *    far-field calls where it is at most 1 GiB (each).  That scratch is given
+ *    back before a call fails with DDA_ERR_OOM.  Device-pointer variants
+ *    (suffix _device) read/write caller-owned device buffers and run on the
+ *    context's stream.
  *  - Errors: every call returns a dda_status; on failure the message is
  *    available from dda_last_error(ctx) and no output buffer is written,
  *    except that dda_solve fills res[] (status per RHS) when it returns

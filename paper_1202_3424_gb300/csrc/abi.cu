@@ -121,6 +121,7 @@ struct dda_ctx {
     size_t h_stage_bytes = 0;
     cudaEvent_t stage_ev = nullptr;
     int tw_len[3] = {0, 0, 0};  // lengths the twiddle tables hold
+    bool field_busy = false;    // a call works in S_FIELD
     Profiler prof;
 
     dda_status fail(dda_status code, const char* fmt, ...) {
@@ -176,6 +177,26 @@ enum Slot {
     S_NSLOTS
 };
 
+// Device memory for m.  Scratch that an earlier call left behind for the next
+// one (S_GREEN, S_FIELD) is given back before a shortage is reported.
+cudaError_t device_alloc(dda_ctx* ctx, DevMem& m, size_t bytes) {
+    bytes = bytes < 256 ? 256 : bytes;
+    m = DevMem{};
+    cudaError_t e = cudaMalloc(&m.p, bytes);
+    for (int kept : {S_GREEN, S_FIELD}) {
+        DevMem& k = ctx->pool[kept];
+        if (e != cudaErrorMemoryAllocation) break;
+        if (&k == &m || k.p == nullptr || (kept == S_FIELD && ctx->field_busy)) continue;
+        cudaGetLastError();
+        cudaFree(k.p);  // (waits for the device)
+        k = DevMem{};
+        e = cudaMalloc(&m.p, bytes);
+    }
+    m.bytes = e == cudaSuccess ? bytes : 0;
+    if (e != cudaSuccess) m.p = nullptr;
+    return e;
+}
+
 dda_status ensure(dda_ctx* ctx, DevMem& m, size_t bytes, bool zero = false) {
     if (m.bytes >= bytes && m.p != nullptr) {
         if (zero) CU(cudaMemsetAsync(m.p, 0, bytes, ctx->stream));
@@ -191,8 +212,7 @@ dda_status ensure(dda_ctx* ctx, DevMem& m, size_t bytes, bool zero = false) {
         cudaGraphExecDestroy(ctx->graph.exec);
         ctx->graph.exec = nullptr;
     }
-    CU(cudaMalloc(&m.p, bytes < 256 ? 256 : bytes));
-    m.bytes = bytes < 256 ? 256 : bytes;
+    CU(device_alloc(ctx, m, bytes));
     if (zero) CU(cudaMemsetAsync(m.p, 0, m.bytes, ctx->stream));
     return DDA_OK;
 }
@@ -201,9 +221,7 @@ dda_status ensure(dda_ctx* ctx, DevMem& m, size_t bytes, bool zero = false) {
 dda_status ensure_scratch(dda_ctx* ctx, DevMem& m, size_t bytes) {
     if (m.bytes >= bytes && m.p != nullptr) return DDA_OK;
     if (m.p) cudaFree(m.p);
-    m = DevMem{};
-    CU(cudaMalloc(&m.p, bytes < 256 ? 256 : bytes));
-    m.bytes = bytes < 256 ? 256 : bytes;
+    CU(device_alloc(ctx, m, bytes));
     return DDA_OK;
 }
 
@@ -1985,11 +2003,13 @@ dda_status nf_box(dda_ctx* ctx, const double* ext, int dims[3], int off[3]) {
     return DDA_OK;
 }
 
-// Gives the field calls' workspace back where it is too large to keep.
+// The field calls' workspace while it is in use; given back after the call
+// where it is too large to keep.
 struct ScratchGuard {
     dda_ctx* ctx;
-    explicit ScratchGuard(dda_ctx* c) : ctx(c) {}
+    explicit ScratchGuard(dda_ctx* c) : ctx(c) { ctx->field_busy = true; }
     ~ScratchGuard() {
+        ctx->field_busy = false;
         if (ctx->pool[S_FIELD].bytes <= kKeepMax) return;
         cudaStreamSynchronize(ctx->stream);
         free_mem(ctx->pool[S_FIELD]);
