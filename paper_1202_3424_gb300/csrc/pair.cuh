@@ -38,15 +38,6 @@ __device__ __forceinline__ P2 pmul(P2 a, f32x2 c, f32x2 y, f32x2 ny) {
 // ---- small DFTs, sign convention exp(SGN * 2 pi i j k / R) ----------------
 template <int R, int SGN> struct PDft;
 
-template <int SGN> struct PDft<2, SGN> {
-    __device__ __forceinline__ static void run(P2* v) {
-        const P2 a = v[0], b = v[1];
-        v[0] = padd(a, b);
-        v[1] = psub(a, b);
-    }
-    __device__ __forceinline__ static void run_half(P2* v) { v[1] = v[0]; }
-};
-
 template <int SGN> struct PDft<3, SGN> {
     __device__ __forceinline__ static void run(P2* v) {
         const f32x2 h = pk(-0.5f, -0.5f);
@@ -146,8 +137,15 @@ template <int SGN> struct PDft<16, SGN> {
             return P2{mul2(q.re, pk(-r2, -r2)), mul2(q.im, pk(-r2, -r2))};
         }
     }
-    // (the product with w16^4 = SGN i of y[2][2] goes into the last DFT's sums)
-    __device__ __forceinline__ static void finish(P2* v, P2 (&y)[4][4]) {
+    __device__ __forceinline__ static void run(P2* v) {
+        P2 y[4][4];
+#pragma unroll
+        for (int n2 = 0; n2 < 4; ++n2) {
+#pragma unroll
+            for (int n1 = 0; n1 < 4; ++n1) y[n2][n1] = v[4 * n1 + n2];
+            PDft<4, SGN>::run(y[n2]);
+        }
+        // (the product with w16^4 = SGN i of y[2][2] goes into the last DFT's sums)
         y[1][1] = w16<1>(y[1][1]);
         y[1][2] = w16<2>(y[1][2]);
         y[1][3] = w16<3>(y[1][3]);
@@ -172,27 +170,6 @@ template <int SGN> struct PDft<16, SGN> {
 #pragma unroll
             for (int k2 = 0; k2 < 4; ++k2) v[k1 + 4 * k2] = z[k2];
         }
-    }
-    __device__ __forceinline__ static void run(P2* v) {
-        P2 y[4][4];
-#pragma unroll
-        for (int n2 = 0; n2 < 4; ++n2) {
-#pragma unroll
-            for (int n1 = 0; n1 < 4; ++n1) y[n2][n1] = v[4 * n1 + n2];
-            PDft<4, SGN>::run(y[n2]);
-        }
-        finish(v, y);
-    }
-    // inputs 8..15 are zero
-    __device__ __forceinline__ static void run_half(P2* v) {
-        P2 y[4][4];
-#pragma unroll
-        for (int n2 = 0; n2 < 4; ++n2) {
-            y[n2][0] = v[n2];
-            y[n2][1] = v[4 + n2];
-            PDft<4, SGN>::run_half(y[n2]);
-        }
-        finish(v, y);
     }
 };
 
@@ -280,7 +257,7 @@ template <int K, bool PAD> __device__ __forceinline__ int exchange_slot(int base
 // to save the two moves, took five wavefronts each where these take one:
 // together a fifth of the slab pass's shared-memory cycles).  tw: the table of
 // a length of `every` times the plan's.
-template <class PL, int DIR, int S = 0> __host__ __device__ constexpr int pair_tw_offset(int stage) {
+template <class PL, int DIR> __host__ __device__ constexpr int pair_tw_offset(int stage) {
     int off = 0;
     for (int s = 1; s < stage; ++s) off += (stage_radix<PL, DIR>(s) - 1) * stage_p<PL, DIR>(s);
     return off;
