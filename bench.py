@@ -198,6 +198,7 @@ def pass_bytes(kind, info, R, ncomp_tables=1):
     if kind.startswith("yx_inv"):             # fused y+x slice pass: U2 and X in, Y out
         return R * (u2 + 2 * vec) + 4 * M + N
     if kind.startswith("slab"):               # y and z transforms over kx slabs: the x-transformed rows, both ways
+        # (the octant once, as for the z pass; the kernel reads a copy nearly twice that size)
         return R * 2 * u1 + oct_
     if kind.startswith("x_fwd"):
         return R * (vec + u1) + 4 * M

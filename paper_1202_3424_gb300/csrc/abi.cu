@@ -171,7 +171,7 @@ enum Slot {
     S_MV_X32, S_MV_Y32, S_GRAD, S_DBETA,
     S_BETADF, S_XDF, S_YDF, S_TUNE, S_IN_U2,
     S_TABLES,  // holds S_BETA64, S_BETA32, S_BETADF, S_W, S_KHAT, S_EPOL
-    S_SCALARS, // holds S_STATE, S_NORM_B, S_NORM_R, S_QSUM, S_TOLREL, S_SCALE, S_COEF, S_OUTER
+    S_SCALARS, // holds S_NORM_B, S_NORM_R, S_STATE, S_TOLREL, S_SCALE, S_COEF, S_OUTER
     S_GREEN,   // scratch of dda_prepare's transforms
     S_FIELD,   // workspace of the near and far field calls
     S_NSLOTS

@@ -98,7 +98,6 @@ cudaError_t launch_einc(int R, int64_t N, const int* lat_of, const Geom& g, doub
 // E_inc at points lat_of[j] of an nx*ny-row lattice, phase origin at (cx, cy, cz) in its index space.
 cudaError_t launch_einc_at(int R, int64_t N, const int* lat_of, int nx, int ny, double cx, double cy, double cz,
                            double kd, const double* khat, const double2* e, double2* E, cudaStream_t s);
-// Near field: target sites into the extended-box vector; E_sca = -y in complex128.
 // Per-site materials (N sites, refractive indices m, ambient index m_amb): the
 // LATTDR tables of upload_tables for R RHS with factors S[r] -- entry s + 1 of RHS
 // r for site s, entry 0 zero -- in FP64, FP32 and double-float, and the absorption
@@ -117,6 +116,7 @@ cudaError_t launch_site_deps(int64_t N, const double2* m, double m_amb, double k
 cudaError_t launch_box_maps(const Geom& g, const int dims[3], int* site_of, int* lat_of, cudaStream_t st);
 cudaError_t launch_box_sites(const Geom& gt, int64_t N, const int* lat_of, const int dims[3], const int off[3],
                              int* box_of, cudaStream_t st);
+// Near field: target sites into the extended-box vector; E_sca = -y in complex128.
 template <typename C>
 cudaError_t launch_scatter_sites(int R, int64_t N, int64_t Ne, const int* box_of, const double2* P, C* Pbox,
                                  cudaStream_t s);

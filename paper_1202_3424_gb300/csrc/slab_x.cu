@@ -9,13 +9,17 @@ namespace dda {
 namespace {
 
 // Radix plan variants of the warp-local rows (XwPlan), by the fused mode of the
-// matvec.  Forward: a plain gather takes the plan with the fewest exchanges
-// through shared memory; the BiCGstab gathers, which hold up to seven operands
-// per point, the one with the fewest points per lane (64 RHS of the 96x64x32
-// ellipsoid 329 us, against 393; 64^3 sphere, 2 RHS 20.5 against 23.7 us).
-// Inverse: the fewest points per lane, but for 192 points, where the plan with
-// three exchanges stays at its shared-memory rate (the ellipsoid in a solve
-// 412 us, against 354 with two exchanges; plain, 32 RHS, 190 against 168).
+// matvec: plan 0 (fewer points per lane) or plan 1 (fewer exchanges through
+// shared memory), us per launch with plan 0 / 1 by row length:
+//                                    128a       192b       256c       512d
+//   forward, plain gather          16.4/14.6   110/114    54/42      55/46
+//   forward, in a solve            19.8/22.7   167/198    68/72      69/-
+//   inverse, plain                 14.3/14.3   184/170    84/71      93/99
+//   inverse, in a solve            20.1/20.9   220/182    86/86      88/103
+// (a 64^3 sphere, 2 RHS; b 96x64x32 ellipsoid, 32 RHS; c 128x48x24, 16 RHS; d
+// 256x48x24, 8 RHS.)  A plain gather takes plan 1 up to 256 points; the BiCGstab
+// gathers, which hold up to seven operands per point, plan 0; the inverse plan 1
+// at 192 and 256 points.  (512 points still gather with plan 0.)
 template <int LX, int MODE> constexpr int kPlanFwd = MODE == 0 && (LX == 128 || LX == 192 || LX == 256) ? 1 : 0;
 template <int LX> constexpr int kPlanInv = LX == 192 || LX == 256 ? 1 : 0;
 
