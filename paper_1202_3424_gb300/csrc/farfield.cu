@@ -24,6 +24,7 @@ constexpr int kFFWarps = 8;
 // Rows a block sums before its totals go to FP64: a bound on the length of the
 // sums in the arithmetic type.
 constexpr int kFFRows = 256;
+constexpr int kFFMaxSmem = 227 * 1024;  // dynamic shared memory a block can have
 
 // n consecutive complex numbers from shared memory, in 16-byte words where they fit
 template <int n, typename C> __device__ __forceinline__ void read_words(C (&v)[n], const C* s) {
@@ -223,10 +224,9 @@ cudaError_t launch_farfield(const Geom& g, const DevTarget& tg, const FarGeom& f
                                  std::min<int64_t>(want, (tg.nrows + kFFWarps - 1) / kFFWarps)));
     const int per_chunk = (tg.nrows + chunks - 1) / chunks;
     auto go = [&](auto kern) -> cudaError_t {
-        if (sm > 48 * 1024) {
-            e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-            if (e != cudaSuccess) return e;
-        }
+        // the limit, not sm: another thread's context may set it between here and the launch
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kFFMaxSmem);
+        if (e != cudaSuccess) return e;
         PROF_BEGIN(st);
         kern<<<dim3(tiles, groups, chunks), kFFWarps * 32, sm, st>>>(P, g.N, tg.rows, tg.row_start, tg.nrows, per_chunk,
                                                                     tg.lat_of, g.nx, g.ny, f, tabs, dirs, kd, F);
