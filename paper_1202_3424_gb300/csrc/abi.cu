@@ -1195,6 +1195,7 @@ dda_status solve_core(dda_ctx* ctx, int R, const dda_opts& o, bool refine, bool 
         for (int r = 0; r < R; ++r) {
             std::memset(&hst[r], 0, sizeof(KState));
             hst[r].maxit = std::max(1, o.maxit - tr[r].iters);
+            if (refine && sizeof(T) == 4 && hact[r]) hst[r].q.near_rel = 0.5 * o.tol * tr[r].bn / tr[r].rn;
         }
         // (the stream is idle here, and every pass of this loop ends with a synchronization)
         CU(cudaMemcpyAsync(dev + sp.state, h + sp.state, sp.p.total - sp.state, cudaMemcpyHostToDevice, s));

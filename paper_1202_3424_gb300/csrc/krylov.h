@@ -21,6 +21,7 @@ struct QmrScalars {
     int lanczos_breakdown;      // v_{n+1}^T v_{n+1} = 0
     double best;                // smallest |r| so far and its iteration (stagnation test)
     int best_iter;
+    double near_rel;            // |r| / |b| below which a lack of progress ends the solve (0: never)
 };
 
 // Per-RHS scalars of one Krylov solve, all FP64, kept on the device.

@@ -153,9 +153,10 @@ def test_slab_pass_where_it_is_not_built(lib):
 
 
 def test_refined_solves_stop_alike_on_either_passes(lib):
-    """Inner solves stop at a third of the tolerance, whichever passes run: the
-    true residual exceeds that by the drift of the FP32 recurrence alone (some
-    sixty products, 2^-24 each, of a solution of the incident field's size: 4e-6)."""
+    """Inner solves stop at a third of the tolerance (QMR, where it makes no
+    progress, at half), whichever passes run: the true residual exceeds that by
+    the drift of the FP32 recurrence alone (some sixty products, 2^-24 each, of
+    a solution of the incident field's size: 4e-6)."""
     ctx = _ctx(lib, sphere_grid(24), 1.5 + 0.02j, 3.0)
     rng = np.random.default_rng(2)
     k = rng.standard_normal((16, 3))
@@ -168,7 +169,30 @@ def test_refined_solves_stop_alike_on_either_passes(lib):
         for solver in ("bicgstab", "bicgstab2", "qmr"):
             res, _, st = ctx.solve(lib.Precision.FP32_REFINED, k, e, want_P=False, tol=tol, maxit=400, solver=solver)
             assert st == 0
-            assert max(r["resid_rel"] for r in res) <= tol / 3 + 4e-6, (on, solver)
+            share = 1 / 2 if solver == "qmr" else 1 / 3
+            assert max(r["resid_rel"] for r in res) <= share * tol + 4e-6, (on, solver)
+    ctx.close()
+
+
+def test_qmr_does_not_stall_below_half_the_tolerance(lib):
+    """QMR's residual levels out above the third of the tolerance that inner
+    solves aim at, for one direction in four here.  Below the half, waiting 40
+    iterations for a new minimum buys nothing: what is left are the few that
+    level out above it (iterations of an unhindered solve: 51 to 63)."""
+    u = ((np.arange(64) - 31.5) / 64) ** 2
+    ctx = _ctx(lib, (u[:, None, None] + u[None, :, None] + u[None, None, :] <= 0.25).astype(np.uint8), 1.5 + 0.02j, 5.0)
+    rng = np.random.default_rng(1)
+    iters = []
+    for _ in range(40):
+        k = rng.standard_normal(3)
+        k /= np.linalg.norm(k)
+        a = np.cross([0.0, 0.0, 1.0], k)
+        a /= np.linalg.norm(a)
+        res, _, st = ctx.solve(lib.Precision.FP32_REFINED, np.stack([k, k]), np.stack([a, np.cross(k, a)]).astype(complex),
+                               want_P=False, tol=1e-5, maxit=2000, solver="qmr")
+        assert st == 0
+        iters.append(max(r["iters"] for r in res))
+    assert sum(i > 80 for i in iters) <= 4, sorted(iters)
     ctx.close()
 
 
