@@ -32,9 +32,9 @@
 // latency and dependent issue at 12 warps per SM (issue 49 %, FP32 pipes 52 %,
 // shared pipe 70 %): 96 registers hold a thread's points, so 168 x 384 threads
 // fill the register file; 512 threads of 128 registers spilled and took 3 % more.
-// Rounds cost besides: phase B deals 16 column groups to 6 warps (Ly 128, Lz 64) or
-// 32 to 12 (128, 128), 89 % of a whole last round, and 12 to 8 (96, 96) or 6 to 4
-// (96, 48), 75 %; and a launch's slabs come in whole waves of the SMs.
+// Whole rounds cost besides: phase B deals 16 column groups to 6 warps (Ly 128, Lz
+// 64) or 32 to 12 (128, 128), which fills 89 % of three rounds, and 12 to 8 (96, 96)
+// or 6 to 4 (96, 48), 75 % of two; and a launch's slabs come in waves of the SMs.
 #pragma once
 
 #include "matvec_impl.cuh"
